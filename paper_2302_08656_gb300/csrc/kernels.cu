@@ -954,7 +954,8 @@ __global__ void __launch_bounds__(256) schur_tile_kernel(DevSched s, DevNum<T> n
 // ------------------------------------------------------------ solve kernels
 
 template <typename T>
-__global__ void solve_pre_kernel(int n, const int* __restrict__ perm, DevNum<T> nm0, const double* __restrict__ b)
+__global__ void solve_pre_kernel(int n, const int* __restrict__ perm, DevNum<T> nm0, const double* __restrict__ b,
+                                 int keep)
 {
     const DevNum<T> nm = nm0.at(blockIdx.y);
     const double* __restrict__ d = nm.d;
@@ -963,7 +964,9 @@ __global__ void solve_pre_kernel(int n, const int* __restrict__ perm, DevNum<T> 
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) {
         int o = perm[k];
-        vec[k] = (T)(d[o] * b[o]);
+        const T v = (T)(d[o] * b[o]);
+        vec[k] = v;
+        if (keep) nm.vin[k] = v;
     }
 }
 
@@ -1548,9 +1551,9 @@ cudaError_t launch_schur_tiles(const DevSched& s, const DevNum<T>& nm, const Fro
 }
 
 template <typename T>
-cudaError_t launch_solve_pre(const DevSched& s, const DevNum<T>& nm, const double* b, int batch, cudaStream_t st)
+cudaError_t launch_solve_pre(const DevSched& s, const DevNum<T>& nm, const double* b, bool keep, int batch, cudaStream_t st)
 {
-    solve_pre_kernel<T><<<dim3(cdiv(s.n, 256), batch), 256, 0, st>>>(s.n, s.perm, nm, b);
+    solve_pre_kernel<T><<<dim3(cdiv(s.n, 256), batch), 256, 0, st>>>(s.n, s.perm, nm, b, keep ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1772,7 +1775,7 @@ cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t b
                                                 int64_t, int, cudaStream_t);                                     \
     template cudaError_t launch_schur_tiles<T>(const DevSched&, const DevNum<T>&, const FrontTile*, int, int,    \
                                                int, cudaStream_t);                                               \
-    template cudaError_t launch_solve_pre<T>(const DevSched&, const DevNum<T>&, const double*, int, cudaStream_t); \
+    template cudaError_t launch_solve_pre<T>(const DevSched&, const DevNum<T>&, const double*, bool, int, cudaStream_t); \
     template cudaError_t launch_solve_post<T>(const DevSched&, const DevNum<T>&, double*, int, cudaStream_t);    \
     template cudaError_t launch_solve_fwd<T>(const DevSched&, const DevNum<T>&, const int*, int, int, int, int,  \
                                              cudaStream_t);                                                      \

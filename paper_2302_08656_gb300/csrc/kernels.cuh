@@ -62,6 +62,7 @@ struct DevNum {
     T* panel = nullptr;               // factor panels
     T* cb = nullptr;                  // contribution blocks
     T* vec = nullptr;                 // step-space solve vector (n)
+    T* vin = nullptr;                 // right-hand side as staged, kept beside vec (TreeSched::fwd_in; n)
     T* cbv = nullptr;                 // solve contribution vectors
     T* f12 = nullptr;                 // assembled pivot rows of panel-class fronts
     DevStat* stat = nullptr;
@@ -81,6 +82,7 @@ struct DevNum {
             r.panel += b * bs_panel;
             r.cb += b * bs_cb;
             r.vec += b * bs_n;
+            r.vin += b * bs_n;
             r.cbv += b * bs_cbv;
             r.f12 += b * bs_f12;
             r.stat += b;
@@ -241,6 +243,8 @@ struct TreeKid {
     int q;                       // tree index of the child, -1 if the child lies below the tree part
     int mc, k;                   // child contribution-block order; its rows landing on parent pivots
     int units;                   // units of the child (0 below the tree part)
+    int nt;                      // ... and its units (ti, 0)
+    int pad;
     int64_t cb_off, rel_ptr;
 };
 struct TreeSched {
@@ -251,10 +255,14 @@ struct TreeSched {
     const TreeUnit* unit = nullptr;    // factorization units in dependency order (front = tree index)
     const TreeUnit* unit_fused = nullptr;   // the same with a forward-solve unit (ti = -1) per front after its level
     int nunits_fused = 0;
+    // 1: every mini front has at most 32 rows, and the fused mode runs the forward step inside the
+    // units (ti, 0) (a lane per row) in the plain unit order; 0: it runs the forward units of unit_fused
+    int fwd_in = 0;
     size_t kid_off = 0;                // shared-memory offset of the children's descriptors (factor kernel)
     const int* inv = nullptr;          // gather maps: parent CB row -> child CB row or -1
     // shared-memory layout parameters (host computed)
     int max_kids = 0, map_w = 0, m_elems = 0;
+    int kid_pitch = 1;           // max_kids rounded up to odd
     int max_F = 0, max_w = 0;
     int fwd_stage = 0;           // 1: forward solve stages the F x w panel in shared memory
     int bwd_stage = 0;           // 1: backward solve stages U12 in shared memory
@@ -325,8 +333,10 @@ cudaError_t launch_solve_fwd_cta(const DevSched& s, const DevNum<T>& nm, const i
 template <typename T>
 cudaError_t launch_solve_bwd_cta(const DevSched& s, const DevNum<T>& nm, const int* fronts, int count,
                                  int max_front, int max_w, int batch, cudaStream_t st);
+// keep: also into nm.vin (the fused refactorization's tree units, TreeSched::fwd_in)
 template <typename T>
-cudaError_t launch_solve_pre(const DevSched& s, const DevNum<T>& nm, const double* b, int batch, cudaStream_t st);
+cudaError_t launch_solve_pre(const DevSched& s, const DevNum<T>& nm, const double* b, bool keep, int batch,
+                             cudaStream_t st);
 template <typename T>
 cudaError_t launch_solve_fwd(const DevSched& s, const DevNum<T>& nm, const int* fronts, int count,
                              int max_front, int max_w, int batch, cudaStream_t st);
@@ -374,8 +384,10 @@ cudaError_t launch_zero_stat(DevStat* stat, cudaStream_t st);
 // caller before the launch); stall = optional test hook (see kkt_debug_stall).
 template <typename T>
 cudaError_t tree_grid(int kind, size_t smem, int* grid);   // kind 0 factor, 1 forward, 2 backward
-// fused != 0: the factor kernel also runs the forward substitution of every tree front (its counter
-// block then holds batch * nq factor counters followed by batch * nq forward counters)
+// fused: the factor kernel also runs the forward substitution of every tree front (its counter block
+// then holds batch * nq factor counters followed by batch * nq forward counters); kFwdUnits: as units
+// of their own (unit_fused), kFwdInside: inside the factorization units (t.fwd_in)
+constexpr int kFwdNone = 0, kFwdUnits = 1, kFwdInside = 2;
 // The tree parts of a group of contexts in one launch; gctr: the group's
 // counter block (ticket, abort flag), cleared by the caller.
 template <typename T>

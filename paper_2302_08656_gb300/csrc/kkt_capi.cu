@@ -494,17 +494,18 @@ kkt_status factor_levels(kkt_ctx* c, DevNum<T>& nm, cudaStream_t st, bool fused 
         }
     }
     if (nq > 0 && with_tree) {
-        const int nu = fused ? c->tsched.nunits_fused : c->tsched.nunits;
-        const int us = fused ? c->tf_split_fused : c->tf_split;
+        const int mode = !fused ? kFwdNone : c->tsched.fwd_in ? kFwdInside : kFwdUnits;
+        const int nu = mode == kFwdUnits ? c->tsched.nunits_fused : c->tsched.nunits;
+        const int us = mode == kFwdUnits ? c->tf_split_fused : c->tf_split;
         if (us > 0) {
             Launch L(c, st, KK_TREE_FACTOR, 1);
             KKT_CUDA(launch_tree_factor<T>(c->sched, c->tsched, nm, B, c->ctr_fac, c->stall, c->opt.spin_limit,
-                                           c->tf_grid, c->tf_smem, fused ? 1 : 0, 0, us, 0, st));
+                                           c->tf_grid, c->tf_smem, mode, 0, us, 0, st));
         }
         if (us < nu) {
             Launch L(c, st, KK_TREE_FACTOR, 1);
             KKT_CUDA(launch_tree_factor<T>(c->sched, c->tsched, nm, B, c->ctr_fac, c->stall, c->opt.spin_limit,
-                                           c->tf_grid_narrow, c->tf_smem, fused ? 1 : 0, us, nu - us, 3, st));
+                                           c->tf_grid_narrow, c->tf_smem, mode, us, nu - us, 3, st));
         }
     }
     return KKT_OK;
@@ -656,7 +657,7 @@ kkt_status solve_t(kkt_ctx* c, const double* b, double* x, cudaStream_t st, int 
     const int B = inst < 0 ? c->batch : 1;
     {
         Launch L(c, st, KK_SOLVE_PRE, 1);
-        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, B, st));
+        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, false, B, st));
     }
     if (inst < 0 && !c->profile && !c->opt.no_graphs) {
         if (!c->g_solve) {
@@ -700,7 +701,7 @@ kkt_status refactor_solve_t(kkt_ctx* c, const double* d_vals, const double* b, d
     }
     {
         Launch L(c, st, KK_SOLVE_PRE, 1);
-        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, B, st));
+        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, c->tsched.fwd_in != 0, B, st));
     }
     if (!c->profile && !c->opt.no_graphs) {
         if (!c->g_ffwd) {
@@ -757,7 +758,7 @@ kkt_status jacobi_t(kkt_ctx* c, const double* b, double* x, cudaStream_t st, int
     (void)nrel;
     {
         Launch L(c, st, KK_SOLVE_PRE, 1);
-        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, 1, st));
+        KKT_CUDA(launch_solve_pre<T>(c->sched, nm, b, false, 1, st));
     }
     {
         const int k = 2 + 3 * c->opt.jacobi_sweeps;
@@ -1153,6 +1154,7 @@ static int64_t plan_bytes(const Analysis& an, int n, int64_t nnz, const kkt_opti
     add(B * n * 8); add(B * n * 8);
     add(B * sp.slots * es); add(B * an.panel_total * es); add(B * std::max<int64_t>(an.cb_total, 1) * es);
     add(B * n * es); add(B * std::max<int64_t>((int64_t)an.rel.size(), 1) * es);
+    if (tp.ts.fwd_in) add(B * n * es);
     add(B * scratch * es);
     add((int64_t)n * (o.restart + 1) * 8); add((int64_t)n * o.restart * 8); add(n * 8); add(n * 8);
     add((int64_t)(kRedScratch + 4096 + 8) * 8);
@@ -1165,7 +1167,7 @@ static int64_t plan_bytes(const Analysis& an, int n, int64_t nnz, const kkt_opti
     const int64_t nq = (int64_t)tp.fr.size();
     add(nq * (int64_t)sizeof(TreeFront)); add((int64_t)tp.kid.size() * (int64_t)sizeof(TreeKid));
     add((int64_t)tp.unit.size() * (int64_t)sizeof(TreeUnit)); add((int64_t)tp.inv.size() * 4);
-    add((int64_t)tp.unit_fused.size() * (int64_t)sizeof(TreeUnit));
+    if (!tp.ts.fwd_in) add((int64_t)tp.unit_fused.size() * (int64_t)sizeof(TreeUnit));
     add((int64_t)tp.bwd_chain.size() * 4); add((int64_t)tp.bwd_chain_ptr.size() * 4);
     add((kCtrHead + 2 * B * nq) * 4); add((kCtrHead + 2 * B * nq) * 4); add(2 * 4);
     add((n + 1) * 4); add(std::max<int64_t>((int64_t)an.rel.size(), 1) * 4);
@@ -1350,6 +1352,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     char* cb = P.take<char>(B * cb_unit * es);
     char* vec = P.take<char>(B * n * es);
     char* cbv = P.take<char>(B * cbv_unit * es);
+    char* vin = tp.ts.fwd_in ? P.take<char>(B * n * es) : nullptr;
     c->panel_scratch = P.take<char>(B * scratch * es);
     c->V = P.take<double>((int64_t)n * (c->opt.restart + 1));
     c->Z = P.take<double>((int64_t)n * c->opt.restart);
@@ -1374,6 +1377,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     TreeFront* tfr = P.take<TreeFront>(nq);
     TreeKid* tkid = P.take<TreeKid>(tp.kid.size());
     TreeUnit* tunit = P.take<TreeUnit>(tp.unit.size());
+    if (tp.ts.fwd_in) tp.unit_fused.clear();               // the forward step runs inside the units
     TreeUnit* tunit_fused = P.take<TreeUnit>(tp.unit_fused.size());
     int* tinv = P.take<int>(tp.inv.size());
     int* tchain = P.take<int>(tp.bwd_chain.size());
@@ -1534,7 +1538,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
         DevNum<float>& nm = c->nf;
         nm.sv = reinterpret_cast<float*>(sv); nm.panel = reinterpret_cast<float*>(panel);
         nm.cb = reinterpret_cast<float*>(cb); nm.vec = reinterpret_cast<float*>(vec);
-        nm.cbv = reinterpret_cast<float*>(cbv); nm.stat = c->stat; nm.pivot_eps = eps; nm.d = c->d_a;
+        nm.cbv = reinterpret_cast<float*>(cbv); nm.vin = reinterpret_cast<float*>(vin); nm.stat = c->stat; nm.pivot_eps = eps; nm.d = c->d_a;
         nm.kcopy = c->kvals;
         nm.keys = keys;
         nm.f12 = reinterpret_cast<float*>(f12);
@@ -1545,7 +1549,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
         DevNum<double>& nm = c->nd;
         nm.sv = reinterpret_cast<double*>(sv); nm.panel = reinterpret_cast<double*>(panel);
         nm.cb = reinterpret_cast<double*>(cb); nm.vec = reinterpret_cast<double*>(vec);
-        nm.cbv = reinterpret_cast<double*>(cbv); nm.stat = c->stat; nm.pivot_eps = eps; nm.d = c->d_a;
+        nm.cbv = reinterpret_cast<double*>(cbv); nm.vin = reinterpret_cast<double*>(vin); nm.stat = c->stat; nm.pivot_eps = eps; nm.d = c->d_a;
         nm.kcopy = c->kvals;
         nm.keys = keys;
         nm.f12 = reinterpret_cast<double*>(f12);

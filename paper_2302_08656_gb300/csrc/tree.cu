@@ -53,19 +53,22 @@ __device__ bool bounded_wait(const int* p, int need, int* abort_flag, long long 
 }
 
 // Bounded wait of warp 0 for the children of a unit: lane l polls the
-// completion counters of children l, l + 32, ... (need = their unit count,
-// or 1 if `one`), so every child is checked in each round while the other
+// completion counters of children l, l + 32, ... (need = their unit count, 1
+// for kWaitOne, their number of units (ti, 0) for kWaitRows), so every child is checked in each round while the other
 // warps of the CTA stay parked at the next barrier. Returns 1 once all are
 // complete, 0 if the wait gave up (the abort flag is then set) or another CTA
 // aborted the kernel. Called by warp 0 only.
-__device__ int warp_wait_kids(const int* done_b, const TreeKid* kids, int nk, bool one, int* abort_flag,
+enum { kWaitUnits = 0, kWaitOne = 1, kWaitRows = 2 };
+__device__ int warp_wait_kids(const int* done_b, const TreeKid* kids, int nk, int what, int* abort_flag,
                               long long limit, const int* extra = nullptr, int extra_need = 0)
 {
     const int lane = threadIdx.x & 31;
     for (long long it = 0;; ++it) {
         bool ok = true;
         for (int c = lane; c < nk; c += 32)
-            if (kids[c].q >= 0 && ld_acquire(done_b + kids[c].q) < (one ? 1 : kids[c].units)) ok = false;
+            if (kids[c].q >= 0 && ld_acquire(done_b + kids[c].q) <
+                                      (what == kWaitOne ? 1 : what == kWaitRows ? kids[c].nt : kids[c].units))
+                ok = false;
         if (extra && lane == 0 && ld_acquire(extra) < extra_need) ok = false;
         if (__all_sync(0xffffffffu, ok)) return 1;
         if ((it & 31) == 31) {
@@ -87,10 +90,14 @@ __device__ int warp_wait_kids(const int* done_b, const TreeKid* kids, int nk, bo
 // happen before it), one thread adds 1 to the counter with a release
 // reduction at GPU scope, which makes them visible to a CTA that acquires the
 // counter.
+__device__ __forceinline__ void red_release(int* counter)
+{
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(counter) : "memory");
+}
 __device__ __forceinline__ void signal_done(int* counter)
 {
     __syncthreads();
-    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(counter) : "memory");
+    if (threadIdx.x == 0) red_release(counter);
 }
 
 // Take the next ticket (or `total` once the kernel was aborted): the abort
@@ -294,11 +301,16 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         const int B = MULTI ? sj->B : B_p;
         int* done = (MULTI ? sj->ctr : ctr) + kCtrHead;
         int* fwd_done = done + (int64_t)B * ts.nq;                 // fused mode: forward-unit counters
-        const TreeUnit* units = fused ? ts.unit_fused : ts.unit;
+        const TreeUnit* units = fused == kFwdUnits ? ts.unit_fused : ts.unit;
         T* M = reinterpret_cast<T*>(smraw);
         const int W = ts.map_w;
         const size_t off_map = align16(sizeof(T) * (size_t)ts.m_elems);
-        int* smap = reinterpret_cast<int*>(smraw + off_map);       // child c: rows at 2cW, columns at (2c+1)W
+        // gather maps: mini-front row i takes row rmap[c W + i] of child c's block, column j column
+        // cmap[j KP + c] (-1: none); columns are the leading index there, so that a warp's ballot over the
+        // children of one column, and a lane's store of its column, meet no bank conflict (KP is odd)
+        const int KP = ts.kid_pitch;
+        int* rmap = reinterpret_cast<int*>(smraw + off_map);
+        int* cmap = rmap + ts.max_kids * W;
         TreeKid* kids = reinterpret_cast<TreeKid*>(smraw + ts.kid_off);
         copy_words(&su, units + (MULTI ? 0 : u0) + ul, 1, tid, 256);
         __syncthreads();
@@ -323,18 +335,22 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         // ---- everything that does not depend on the children
         for (int e = tid; e < Fr * Fc; e += 256) M[e] = T(0);
         copy_words(kids, ts.kid + d.kid_begin, nk, tid, 256);
-        for (int e = tid; e < nk * W; e += 256) {
-            const int c = e / W, i = e - c * W;
-            int vr = -1, vc = -1;
-            if (i >= w) {
-                const int* inv = ts.inv + d.inv_off + (int64_t)c * m;
-                if (i - w < nr) vr = inv[i0 + i - w];
-                if (i - w < nc) vc = inv[j0 + i - w];
-            }
-            smap[2 * c * W + i] = vr;
-            smap[(2 * c + 1) * W + i] = vc;
-        }
         __syncthreads();
+        for (int c = ty; c < nk; c += 8) {                         // a warp per child
+            const int* inv = ts.inv + d.inv_off + (int64_t)c * m - w;
+            for (int i = tx; i < W; i += 32) {
+                if (i < Fr) rmap[c * W + i] = i >= w ? inv[i0 + i] : -1;
+                if (i < Fc) cmap[i * KP + c] = i >= w ? inv[j0 + i] : -1;
+            }
+            __syncwarp();
+            const int k = kids[c].k;                               // child rows t < k land on pivots
+            const int* rl = s.rel + kids[c].rel_ptr;
+            for (int tt = tx; tt < k; tt += 32) {
+                const int r = rl[tt];
+                rmap[c * W + r] = tt;
+                cmap[r * KP + c] = tt;
+            }
+        }
         for (int64_t e = d.asm_begin + tid; e < d.asm_end; e += 256) {
             const int pos = s.asm_pos[e];
             const int bc = pos / F, a = pos - bc * F;
@@ -342,17 +358,11 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             const int lc = bc < w ? bc : ((unsigned)(bc - w - j0) < (unsigned)nc ? bc - j0 : -1);
             if (lr >= 0 && lc >= 0) M[lr + lc * Fr] = nm.sv[s.asm_src[e]];
         }
-        for (int c = ty; c < nk; c += 8) {                         // child rows t < k land on pivots
-            const int k = kids[c].k;
-            const int* rl = s.rel + kids[c].rel_ptr;
-            for (int tt = tx; tt < k; tt += 32) {
-                const int r = rl[tt];
-                smap[2 * c * W + r] = tt;
-                smap[(2 * c + 1) * W + r] = tt;
-            }
-        }
         // static-pivot floor (the scaling kernel's max |D K D|), loaded before the wait
         const T floorT = (T)(nm.pivot_eps * __longlong_as_double((long long)nm.stat->amax_bits));
+        const bool fwd_here = !MULTI && fused == kFwdInside && ut.tj == 0;   // warp 0's forward step below
+        T xf = T(0);
+        if (fwd_here && tid < w) xf = nm.vin[d.first + tid];       // w <= 32; vin: the lead unit overwrites vec
         // ---- wait for the children (bounded; lane l of warp 0 polls children l, l + 32)
         if (tid == 0) {
             s_ok = 1;
@@ -361,9 +371,9 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 *stall = 0;
             }
         }
-        __syncthreads();
-        if (s_ok && tid < 32) {
-            const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, kids, nk, false, ctr + 1, limit);
+        __syncwarp();
+        if (tid < 32 && s_ok) {
+            const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, kids, nk, kWaitUnits, ctr + 1, limit);
             if (tid == 0) s_ok = ok;
         }
         __syncthreads();
@@ -372,37 +382,55 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             break;
         }
         // ---- children's contributions, in child order for every entry; each
-        // thread holds four entries of one row and keeps up to 16 loads in flight
-        for (int i = tx; i < Fr; i += 32)
+        // thread holds four entries of one row and keeps up to 16 loads in
+        // flight. A warp visits, column by column, only the children that
+        // reach the column (a ballot over the children): fronts of the lower
+        // tree levels have up to 37 children of a few rows each, and testing
+        // every child for every entry took most of a unit's instructions
+        // there (70k buses, with the forward step below: FP32 step 1820 ->
+        // 1726 us, FP64, whose adds of nothing cost pipe time, 3190 -> 2924).
+        for (int ib = 0; ib < Fr; ib += 32)
             for (int jb = ty; jb < Fc; jb += 32) {
+                const int i = ib + tx;
+                const bool in = i < Fr;
                 T acc[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = jb + 8 * k < Fc ? M[i + (jb + 8 * k) * Fr] : T(0);
-                for (int c = 0; c < nk; c += 4) {
-                    T v[4][4];
-                    unsigned valid = 0u;
+                for (int k = 0; k < 4; ++k) acc[k] = in && jb + 8 * k < Fc ? M[i + (jb + 8 * k) * Fr] : T(0);
+                for (int h = 0; h < nk; h += 32) {
+                    unsigned mk[4];                                // children h + bit that reach column jb + 8 k
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const int cc = c + g;
-                        const int sr = cc < nk ? smap[2 * cc * W + i] : -1;
+                    for (int k = 0; k < 4; ++k)
+                        mk[k] = __ballot_sync(0xffffffffu, jb + 8 * k < Fc && h + tx < nk &&
+                                                               cmap[(jb + 8 * k) * KP + h + tx] >= 0);
+                    while (mk[0] | mk[1] | mk[2] | mk[3]) {
+                        T v[4][4];
+                        unsigned valid = 0u;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int j = jb + 8 * k;
-                            const int sc = (cc < nk && j < Fc) ? smap[(2 * cc + 1) * W + j] : -1;
-                            const bool ok = sr >= 0 && sc >= 0;
-                            v[g][k] = ok ? __ldcg(nm.cb + kids[cc].cb_off + sr + (int64_t)sc * kids[cc].mc) : T(0);
-                            valid |= ok ? (1u << (4 * g + k)) : 0u;
-                        }
+                        for (int g = 0; g < 4; ++g)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                v[g][k] = T(0);
+                                if (mk[k]) {
+                                    const int c = h + __ffs(mk[k]) - 1;
+                                    mk[k] &= mk[k] - 1u;
+                                    const int sr = in ? rmap[c * W + i] : -1;
+                                    const int sc = cmap[(jb + 8 * k) * KP + c];
+                                    if (sr >= 0) {
+                                        v[g][k] = __ldcg(nm.cb + kids[c].cb_off + sr + (int64_t)sc * kids[c].mc);
+                                        valid |= 1u << (4 * g + k);
+                                    }
+                                }
+                            }
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                if (valid & (1u << (4 * g + k))) acc[k] += v[g][k];
                     }
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (valid & (1u << (4 * g + k))) acc[k] += v[g][k];
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (jb + 8 * k < Fc) M[i + (jb + 8 * k) * Fr] = acc[k];
+                    if (in && jb + 8 * k < Fc) M[i + (jb + 8 * k) * Fr] = acc[k];
             }
         __syncthreads();
         // ---- w pivot steps of right-looking elimination without pivoting, one
@@ -520,7 +548,16 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 for (int i = w + tid; i < Fr; i += 256) M[i + (w - 1) * Fr] *= s_rinv[w - 1];
             __syncthreads();
         }
-        // ---- results: pivot block (lead unit), L21 rows (tj == 0), U12 columns (ti == 0), CB tile
+        // ---- results: the CB tile, all that the parent's units wait for, first
+        // and signalled by warp 7 (the panel too where forward units read it);
+        // then pivot block (lead unit), L21 rows (tj == 0), U12 columns (ti == 0)
+        T* C = nm.cb + d.cb_off;
+        for (int c = ty; c < nc; c += 8)
+            for (int r = tx; r < nr; r += 32) C[(i0 + r) + (int64_t)(j0 + c) * m] = M[(w + r) + (w + c) * Fr];
+        if (fused != kFwdUnits) {
+            __syncthreads();
+            if (tid == 224) red_release(done + (int64_t)b * ts.nq + q);
+        }
         T* pan = nm.panel + d.panel_off;
         if (lead)
             for (int c = ty; c < w; c += 8)
@@ -533,10 +570,44 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             for (int c = ty; c < nc; c += 8)
                 for (int a = tx; a < w; a += 32) U12[a + (int64_t)(j0 + c) * w] = M[a + (w + c) * Fr];
         }
-        T* C = nm.cb + d.cb_off;
-        for (int c = ty; c < nc; c += 8)
-            for (int r = tx; r < nr; r += 32) C[(i0 + r) + (int64_t)(j0 + c) * m] = M[(w + r) + (w + c) * Fr];
-        signal_done(done + (int64_t)b * ts.nq + q);
+        if (fused == kFwdUnits) {
+            signal_done(done + (int64_t)b * ts.nq + q);
+        } else if (fwd_here && ty == 0) {
+            // forward step of the stripe (lane -> row of the mini front): the
+            // operations of fwd_unit in its order. The children's vectors are
+            // complete by now as a rule (their units finished before this
+            // one's wait ended), and the parent waits for this step only
+            // after its own elimination, so it is off the critical path. A
+            // unit of its own per front (8.6 us each, as long as a
+            // factorization unit) took 40 % of the CTAs' time on the wide
+            // levels.
+            const int ok = warp_wait_kids(fwd_done + (int64_t)b * ts.nq, kids, nk, kWaitRows, ctr + 1, limit);
+            if (ok) {
+                for (int c0 = 0; c0 < nk; c0 += 8) {
+                    T cv[8];
+                    unsigned has = 0u;
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) {
+                        const int sr = c0 + g < nk && tx < Fr ? rmap[(c0 + g) * W + tx] : -1;
+                        cv[g] = sr >= 0 ? __ldcg(nm.cbv + kids[c0 + g].rel_ptr + sr) : T(0);
+                        has |= sr >= 0 ? 1u << g : 0u;
+                    }
+#pragma unroll
+                    for (int g = 0; g < 8; ++g)
+                        if (has & (1u << g)) xf += cv[g];
+                }
+                for (int p = 0; p < w; ++p) {
+                    const T xp = __shfl_sync(0xffffffffu, xf, p);
+                    if (tx > p && tx < Fr) xf -= M[tx + p * Fr] * xp;
+                }
+                if (lead && tx < w) nm.vec[d.first + tx] = xf;
+                if (tx >= w && tx < Fr) nm.cbv[d.rel_ptr + i0 + tx - w] = xf;
+                __syncwarp();
+                if (tx == 0) red_release(fwd_done + (int64_t)b * ts.nq + q);
+            } else if (tx == 0) {
+                atomicExch(&nm.stat->timeout, 1);                  // the abort flag is set: the next ticket ends it
+            }
+        }
     }
 }
 
@@ -668,7 +739,7 @@ __device__ bool fwd_unit(const DevSched& s, const TreeSched& ts, const DevNum<T>
             for (int tt = tid; tt < kids[c].mc; tt += NT) spos[s_cut[c] + tt] = rl[tt];
         }
     if (tid < 32) {
-        const int ok = warp_wait_kids(done_b, kids, nk, true, abort_flag, limit, fused ? fac_done + q : nullptr,
+        const int ok = warp_wait_kids(done_b, kids, nk, kWaitOne, abort_flag, limit, fused ? fac_done + q : nullptr,
                                       d.units);
         if (tid == 0) *s_ok = ok;
     }
@@ -898,7 +969,7 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
         // the bottom front waits for its children in the tree part while its
         // share is in flight
         if (tid < 32) {
-            const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, kb[0], dd[0].kid_end - dd[0].kid_begin, true,
+            const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, kb[0], dd[0].kid_end - dd[0].kid_begin, kWaitOne,
                                           ctr + 1, limit);
             if (tid == 0) s_ok = ok;
         }
@@ -1058,7 +1129,7 @@ __global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts,
             if (k == k0 && tid < 32) {
                 TreeKid par{};
                 par.q = dd[ds].parent;
-                const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, &par, 1, true, ctr + 1, limit);
+                const int ok = warp_wait_kids(done + (int64_t)b * ts.nq, &par, 1, kWaitOne, ctr + 1, limit);
                 if (tid == 0) s_ok = ok;
             }
             __syncthreads();
@@ -1179,9 +1250,10 @@ cudaError_t launch_tree_factor(const DevSched& s, const TreeSched& t, const DevN
 {
     const int g = std::min<long long>(grid, (long long)nu * batch);
     if (g <= 0) return cudaSuccess;
-    if ((fused ? t.unit_fused : t.unit) == nullptr || t.fr == nullptr || t.kid == nullptr)
+    if ((fused == kFwdUnits ? t.unit_fused : t.unit) == nullptr || t.fr == nullptr || t.kid == nullptr)
         return cudaErrorInvalidValue;                         // schedule not uploaded: never launch on it
-    if (u0 < 0 || nu < 0 || u0 + nu > (fused ? t.nunits_fused : t.nunits) || (tick != 0 && tick != 3))
+    if (fused == kFwdInside && (!t.fwd_in || !nm.vin)) return cudaErrorInvalidValue;
+    if (u0 < 0 || nu < 0 || u0 + nu > (fused == kFwdUnits ? t.nunits_fused : t.nunits) || (tick != 0 && tick != 3))
         return cudaErrorInvalidValue;
     tree_factor_entry<false>((const T*)nullptr)<<<g, 256, smem, st>>>(s, t, nm, batch, ctr, stall, spin_limit, fused, u0, nu, tick,
                                                        nullptr, nullptr, 0);

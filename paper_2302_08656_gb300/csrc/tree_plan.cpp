@@ -78,6 +78,7 @@ void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
                 k.mc = an.sn_front[ch] - (an.sn_first[ch + 1] - an.sn_first[ch]);
                 k.k = an.cb_split[ch];
                 k.units = k.q >= 0 ? tp.fr[k.q].units : 0;
+                k.nt = k.q >= 0 ? tp.fr[k.q].nt : 0;
                 k.cb_off = an.cb_off[ch];
                 k.rel_ptr = an.rel_ptr[ch];
                 tp.kid.push_back(k);
@@ -138,6 +139,8 @@ void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
     }
     ts.nunits_fused = (int)tp.unit_fused.size();
     ts.max_kids = std::max(ts.max_kids, 1);
+    ts.kid_pitch = ts.max_kids | 1;
+    ts.fwd_in = ts.map_w <= 32 ? 1 : 0;
     ts.fwd_stage = (size_t)ts.max_fw * es <= kStageLimit ? 1 : 0;
     ts.bwd_stage = 2 * (size_t)ts.max_wm * es <= kStageLimit ? 1 : 0;   // two fronts staged at a time
     // forward chains: the children's entries of the largest front's children
@@ -166,7 +169,8 @@ void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
 
 
 // factor kernel: mini front and gather maps, or (forward units of the fused
-// mode) the forward unit's arrays; the children's descriptors after both
+// mode, where the forward step is not inside the factorization units) the
+// forward unit's arrays; the children's descriptors after both
 static size_t fwd_arrays(const TreeSched& t, size_t es)
 {
     return es * ((size_t)t.max_F + (t.fwd_stage ? (size_t)t.max_fw : (size_t)t.max_w * t.max_w) + kTreeStage) +
@@ -175,8 +179,8 @@ static size_t fwd_arrays(const TreeSched& t, size_t es)
 
 size_t tree_kid_offset(const TreeSched& t, size_t es)
 {
-    const size_t fac = align16(es * (size_t)t.m_elems) + align16(sizeof(int) * 2 * (size_t)t.max_kids * t.map_w);
-    return align16(std::max(fac, fwd_arrays(t, es)));
+    const size_t fac = align16(es * (size_t)t.m_elems) + align16(sizeof(int) * ((size_t)t.max_kids + t.kid_pitch) * t.map_w);
+    return align16(t.fwd_in ? fac : std::max(fac, fwd_arrays(t, es)));
 }
 
 size_t tree_factor_smem(const TreeSched& t, size_t es)
