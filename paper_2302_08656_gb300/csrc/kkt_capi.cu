@@ -237,7 +237,7 @@ size_t elem_size(int precision) { return precision == KKT_FP32_IR ? 4 : 8; }
 constexpr size_t kSmemLimit = 220 * 1024;
 
 // Classify fronts per level and lay out the launch lists.
-void build_levels(const Analysis& an, size_t es, int nlev, std::vector<LevelGroup>& levels,
+void build_levels(const Analysis& an, size_t es, int nlev, int batch, std::vector<LevelGroup>& levels,
                   std::vector<int>& front_ids, std::vector<FrontTile>& tiles, int64_t& scratch_stride,
                   int& max_panel_global, std::vector<int64_t>& inv_off, std::vector<int>& inv,
                   std::vector<int64_t>& f12_off, int64_t& f12_total)
@@ -273,10 +273,14 @@ void build_levels(const Analysis& an, size_t es, int nlev, std::vector<LevelGrou
                 cmax = std::max(cmax, F);
             }
         }
-        // a warp per front pays only when the level has enough fronts to fill
-        // the GPU; on narrow levels a lone warp cannot hide latency, so small
-        // fronts go to the CTA kernels as well
-        if ((int)wl.size() < kWarpLevelMin) {
+        // a warp per front pays only when the level has enough fronts, over
+        // all instances of a batch, to fill the GPU; on narrow levels a lone
+        // warp cannot hide latency, so small fronts go to the CTA kernels as
+        // well. Counted per instance, the levels of 40 to 385 fronts of a
+        // batch of 64 took the CTA kernels (two launches each with the
+        // forward step): step of 64 x 2,000 buses FP32 1971 us, over all
+        // instances 1352 us.
+        if ((int64_t)wl.size() * batch < kWarpLevelMin) {
             for (int s : wl) cmax = std::max(cmax, an.sn_front[s]);
             cl.insert(cl.begin(), wl.begin(), wl.end());
             wl.clear();
@@ -1198,7 +1202,7 @@ kkt_status kkt_plan(int32_t n, const int32_t* h_rowptr, const int32_t* h_colidx,
         int64_t f12_total = 0;
         TreePlan tp;
         build_tree(an, o.tree_min_fronts, elem_size(o.precision), tp);
-        build_levels(an, elem_size(o.precision), tp.split, lv, fids, tiles, stride, mpg, inv_off, inv, f12_off,
+        build_levels(an, elem_size(o.precision), tp.split, 1, lv, fids, tiles, stride, mpg, inv_off, inv, f12_off,
                      f12_total);
         SellPlan sp;
         build_sell(n, h_rowptr, h_colidx, kSellWindow, sp);
@@ -1291,7 +1295,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
         // instance: it stays level-launched once fronts x batch reach the threshold
         const int per_instance = (c->opt.tree_min_fronts + batch - 1) / batch;
         build_tree(c->an, per_instance, elem_size(c->opt.precision), tp);
-        build_levels(c->an, elem_size(c->opt.precision), tp.split, c->levels, fids, tiles, c->scratch_stride,
+        build_levels(c->an, elem_size(c->opt.precision), tp.split, batch, c->levels, fids, tiles, c->scratch_stride,
                      c->max_panel_global, inv_off, inv, f12_off, f12_total);
         // K's per-refactor copies live in the sliced layout: the assembly reads them at slots
         build_sell(n, h_rowptr, h_colidx, kSellWindow, sp);
