@@ -549,4 +549,44 @@ void build_sell(int n, const int* rowptr, const int* colidx, int window, SellPla
         }
 }
 
+// A slice wider than kSellSegment slots is cut into up to kSellWarps
+// contiguous segments, a warp each, all in one block. Slices of most segments
+// come first (their blocks start first), and the warps that a block has left
+// take slices of one segment.
+void segment_sell(SellPlan& out)
+{
+    std::vector<std::vector<int>> by(kSellWarps + 1);
+    for (int s = 0; s < out.nslices; ++s) {
+        const int width = (int)((out.off[s + 1] - out.off[s]) / 32);
+        by[std::max(1, std::min(kSellWarps, (width + kSellSegment - 1) / kSellSegment))].push_back(s);
+    }
+    out.task.clear();
+    int used = 0, most = 1;                                       // warps of the open block
+    size_t one = 0;
+    auto put = [&](int s, int nseg) {
+        const int width = (int)((out.off[s + 1] - out.off[s]) / 32), len = (width + nseg - 1) / nseg;
+        for (int g = 0; g < nseg; ++g) {
+            const int a = std::min(width, g * len), b = std::min(width, a + len);
+            out.task.insert(out.task.end(), {s, (int)(out.off[s] / 32) + a, b - a, g | nseg << 8});
+        }
+        used += nseg;
+        most = std::max(most, nseg);
+    };
+    auto close = [&]() {
+        while (used < kSellWarps && one < by[1].size()) put(by[1][one++], 1);
+        for (; used < kSellWarps; ++used) out.task.insert(out.task.end(), {-1, 0, 0, 255 | 1 << 8});
+        for (size_t w = out.task.size() - 4 * kSellWarps; w < out.task.size(); w += 4) out.task[w + 3] |= most << 16;
+        used = 0;
+        most = 1;
+    };
+    for (int nseg = kSellWarps; nseg > 1; --nseg)
+        for (int s : by[nseg]) {
+            if (used + nseg > kSellWarps) close();
+            put(s, nseg);
+        }
+    if (used) close();
+    while (one < by[1].size()) close();
+    out.nblocks = (int)(out.task.size() / (4 * kSellWarps));
+}
+
 }  // namespace kktgb

@@ -81,11 +81,25 @@ struct SellPlan {
     std::vector<int> ci;              // slots: column index, -1 for padding
     std::vector<int> src;             // slots: CSR position of the entry, -1 for padding
     std::vector<int> csr2sell;        // nnz: slot of each CSR position
+    // segmented form: work of the kernels' warps, kSellWarps per block: {slice,
+    // first slot / 32, slots per lane, segment | segments << 8 | most segments
+    // of a slice in this block << 16}; a warp without work has slice -1 and
+    // segment 255. Empty (nblocks = 0) where a warp takes a whole slice.
+    std::vector<int> task;            // 4 ints per warp
+    int nblocks = 0;
 };
 
 constexpr int kSellWindow = 4096;
+constexpr int kSellWarps = 8;         // warps per block of the kernels on the sliced copy
+// Segmented form up to this many slices, over all instances: about the warps
+// that the chip holds of these kernels (25,000 buses, 5,438 slices: 5 % of a
+// step faster; 70,000, 14,875 slices: 1 to 2 % slower).
+constexpr int kSellSegmentWarps = 8192;
+constexpr int kSellSegment = 16;      // slots of a warp's segment, unless the slice has more than 8 of them
 
 void build_sell(int n, const int* rowptr, const int* colidx, int window, SellPlan& out);
+// The segmented form of a plan (SellPlan::task).
+void segment_sell(SellPlan& out);
 
 // Quotient-graph minimum-degree ordering (exact external degrees, element
 // absorption). order[k] = node eliminated k-th.

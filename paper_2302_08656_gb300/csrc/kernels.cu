@@ -10,6 +10,8 @@
 // the updates grouped by subtree.
 #include "kernels.cuh"
 
+#include "analysis.hpp"
+
 #include <math.h>
 
 namespace kktgb {
@@ -103,14 +105,29 @@ __device__ __forceinline__ int pow2_inv_sqrt_exp(unsigned long long rb)
 
 // ---------------------------------------------------------- equilibration
 
-// Every pass over K runs on its sliced copy (SellPlan): a warp per slice of 32
-// rows, a lane per row, the row's entries k = 0, 1, ... at slots
-// off + 32 k + lane (coalesced across the warp). Row maxima and row sums are
-// then formed by one lane in sequence, with no cross-lane reduction: on this
-// GPU an FP64 warp instruction costs the FP64 pipe the same whether 32 lanes or
-// one do useful work, so the eight-lanes-per-row layout with shuffle sums spent
-// most of its FP64 issue on the reductions.
-constexpr int kSellWarps = 8;                      // slices per 256-thread block
+// Every pass over K runs on its sliced copy (SellPlan): a lane per row, the
+// row's entries k = 0, 1, ... at slots off + 32 k + lane (coalesced across the
+// warp). Row maxima and row sums are then formed with no cross-lane reduction:
+// on this GPU an FP64 warp instruction costs the FP64 pipe the same whether 32
+// lanes or one do useful work, so the eight-lanes-per-row layout with shuffle
+// sums spent most of its FP64 issue on the reductions.
+//
+// A slot costs a chain of two dependent loads (key or value and column, then
+// the gather); a lane loads kSellChunk slots in one round. Where the slices fit
+// the chip at once, a pass takes as long as its longest slice: 52 to 64 slots,
+// 7 rounds of about 2 us, on grids of 200 to 70,000 buses alike, while the mean
+// row has 10. There (kSellSegmentWarps) a slice is cut into segments of
+// kSellSegment slots, a warp each in one block (SellPlan::task; SEG below).
+// Maxima do not depend on the order; a row sum passes from segment to segment
+// through shared memory, so its terms are added in CSR order as before. One
+// pass at 200 buses: 16 -> 5 us; refactor_refine 200 buses FP64 345 -> 315 us,
+// 2,003 FP32 409 -> 372, 9,973 FP64 1071 -> 1021, 25,000 FP32 1008 -> 957.
+// Larger systems and batches keep a warp per slice: there the passes are bound
+// by the gathers' throughput (a scattered 32-lane gather takes about 32 cycles
+// of the SM's L1), and the segments' extra warps cost 2 to 5 % of a step. For
+// the same reason the unsegmented equilibration is held to 48 registers, 5
+// CTAs per SM (4: 2 % of the step of 64 x 2,000 buses).
+constexpr int kSellChunk = 8;
 constexpr unsigned kKeySpecial = 0xffffu;          // subnormal, infinite or NaN entry
 
 // Exponent key of |k|: 0 for zero, (E << 1) | (mantissa != 0) for a normal
@@ -124,11 +141,52 @@ __device__ __forceinline__ unsigned exp_key(double k)
     return (E << 1) | ((b & 0x000fffffffffffffull) != 0ull ? 1u : 0u);
 }
 
-// Slots a lane loads ahead in the sliced kernels: its next kSellChunk keys
-// (or values) and column indices are loaded first, then the kSellChunk
-// gathers, then the arithmetic, so that every lane keeps that many independent
-// loads in flight instead of walking one key -> column -> gather chain at a time.
-constexpr int kSellChunk = 8;
+// A warp's share of a pass: slots o0, o0 + 32, ... < o1 of a lane (one segment
+// of the lane's row).
+struct SellSeg {
+    int slice, seg, nseg, most;                    // most: segments of the block's longest slice
+    int64_t o0, o1;
+    __device__ bool last() const { return seg == nseg - 1; }
+};
+template <bool SEG>
+__device__ __forceinline__ SellSeg sell_seg(const DevSched& s, int wid, int lane)
+{
+    if (!SEG) {
+        const int slice = blockIdx.x * kSellWarps + wid;
+        if (slice >= s.nslices) return SellSeg{-1, 255, 1, 1, 0, 0};
+        return SellSeg{slice, 0, 1, 1, s.sell_off[slice] + lane, s.sell_off[slice + 1]};
+    }
+    const int4 t = s.sell_task[blockIdx.x * kSellWarps + wid];
+    SellSeg g;
+    g.slice = t.x;
+    g.seg = t.w & 255;
+    g.nseg = (t.w >> 8) & 255;
+    g.most = t.w >> 16;
+    g.o0 = 32 * (int64_t)t.y + lane;
+    g.o1 = g.o0 + 32 * (int64_t)t.z;
+    return g;
+}
+// A sum over the slots of each row in CSR order: segment after segment, each
+// warp adding its terms (add) to what the segment before it left. Every thread
+// of the block calls it; the row's sum is in the last segment's warp.
+template <bool SEG, typename F>
+__device__ __forceinline__ double sell_sum(const SellSeg& g, int wid, int lane, double (*carry)[32], F&& add)
+{
+    double acc = 0.0;
+    if (!SEG) {
+        add(acc);
+        return acc;
+    }
+    for (int p = 0; p < g.most; ++p) {
+        if (g.seg == p) {
+            if (p > 0) acc = carry[wid - 1][lane];
+            add(acc);
+            if (!g.last()) carry[wid][lane] = acc;
+        }
+        if (p + 1 < g.most) __syncthreads();
+    }
+    return acc;
+}
 
 // One Ruiz iteration, r_i = max_j |d_i k_ij d_j|, d_i <- d_i 2^round(-log2(r_i)/2),
 // integer-only: every d is a power of two, so |d_i k_ij d_j| is |k_ij| with
@@ -144,7 +202,8 @@ constexpr int kSellChunk = 8;
 // reading din and writes 1 to din as well as the new d to dout. An iteration
 // that changes no d_i leaves dout equal to din, bit for bit, so both buffers
 // already hold the fixed point and every later iteration returns at once.
-__global__ void __launch_bounds__(256) ruiz_sell_kernel(DevSched s, const double* __restrict__ v, int64_t bs_nnz,
+template <bool SEG>
+__global__ void __launch_bounds__(256, SEG ? 1 : 5) ruiz_sell_kernel(DevSched s, const double* __restrict__ v, int64_t bs_nnz,
                                                         double* kcopy, unsigned short* keys, int64_t bs_slot,
                                                         double* din, double* __restrict__ dout, DevStat* stat,
                                                         int it, int load_only)
@@ -156,15 +215,17 @@ __global__ void __launch_bounds__(256) ruiz_sell_kernel(DevSched s, const double
     keys += (int64_t)inst * bs_slot;
     din += (int64_t)inst * s.n;
     dout += (int64_t)inst * s.n;
-    const int lane = threadIdx.x & 31;
-    const int slice = blockIdx.x * kSellWarps + (threadIdx.x >> 5);
-    int changed = 0;
-    if (slice < s.nslices) {
-        const int row = s.sell_row[slice * 32 + lane];
-        const int64_t o0 = s.sell_off[slice] + lane, o1 = s.sell_off[slice + 1];
-        const int ei = (row >= 0 && it > 0) ? exp_of_pow2(din[row]) : 0;
-        unsigned m = 0u;
-        bool special = false;
+    constexpr int kAhead = SEG ? kSellSegment : kSellChunk;
+    __shared__ unsigned s_m[kSellWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const SellSeg g = sell_seg<SEG>(s, wid, lane);
+    const int64_t o0 = g.o0, o1 = g.o1;
+    int changed = 0, row = -1, ei = 0;
+    unsigned m = 0u;
+    bool special = false;
+    if (g.slice >= 0) {
+        row = s.sell_row[g.slice * 32 + lane];
+        ei = (row >= 0 && it > 0) ? exp_of_pow2(din[row]) : 0;
         if (it == 0) {
             for (int64_t ob = o0; ob < o1; ob += 32 * kSellChunk) {
                 int src[kSellChunk];
@@ -189,21 +250,21 @@ __global__ void __launch_bounds__(256) ruiz_sell_kernel(DevSched s, const double
                 }
             }
         } else {
-            for (int64_t ob = o0; ob < o1; ob += 32 * kSellChunk) {
-                unsigned key[kSellChunk];
-                int c[kSellChunk];
+            for (int64_t ob = o0; ob < o1; ob += 32 * kAhead) {
+                unsigned key[kAhead];
+                int c[kAhead];
 #pragma unroll
-                for (int u = 0; u < kSellChunk; ++u) {
+                for (int u = 0; u < kAhead; ++u) {
                     const int64_t o = ob + 32 * u;
                     key[u] = o < o1 ? keys[o] : 0u;
                     c[u] = o < o1 ? s.sell_ci[o] : -1;
                 }
-                int ej[kSellChunk];
+                int ej[kAhead];
 #pragma unroll
-                for (int u = 0; u < kSellChunk; ++u)
+                for (int u = 0; u < kAhead; ++u)
                     ej[u] = (key[u] != 0u && key[u] != kKeySpecial) ? exp_of_pow2(din[c[u]]) : 0;
 #pragma unroll
-                for (int u = 0; u < kSellChunk; ++u) {
+                for (int u = 0; u < kAhead; ++u) {
                     if (key[u] == 0u) continue;
                     if (key[u] == kKeySpecial) { special = true; continue; }
                     const int E = (int)(key[u] >> 1) + ei + ej[u];
@@ -213,11 +274,24 @@ __global__ void __launch_bounds__(256) ruiz_sell_kernel(DevSched s, const double
                 }
             }
         }
+    }
+    if (SEG && g.most > 1) {                                       // a row's segments (uniform over the block)
+        s_m[wid][lane] = m | (special ? 0x80000000u : 0u);
+        __syncthreads();
+        if (g.seg == 0)
+            for (int q = 1; q < g.nseg; ++q) {
+                const unsigned mq = s_m[wid + q][lane];
+                special = special || (mq >> 31);
+                m = max(m, mq & 0x7fffffffu);
+            }
+    }
+    if (g.seg == 0) {
         if (row >= 0 && !load_only) {
             int e = 0;
             if (special) {
                 unsigned long long mk = 0ull;
-                for (int64_t o = o0; o < o1; o += 32) {
+                const int64_t r1 = s.sell_off[g.slice + 1];        // the whole row
+                for (int64_t o = o0; o < r1; o += 32) {
                     const int c = s.sell_ci[o];
                     if (c < 0) continue;
                     const int ej = it > 0 ? exp_of_pow2(din[c]) : 0;
@@ -244,19 +318,20 @@ __global__ void __launch_bounds__(256) ruiz_sell_kernel(DevSched s, const double
 // D K D in factor precision (sliced layout: the assembly reads it through
 // asm_src), max |D K D| (static-pivot reference) and ||K||_inf, whose row sums
 // each lane forms in CSR order.
-template <typename T>
+template <typename T, bool SEG>
 __global__ void __launch_bounds__(256) scale_sell_kernel(DevSched s, DevNum<T> nm0)
 {
     const DevNum<T> nm = nm0.at(blockIdx.y);
     const double* __restrict__ d = nm.d;
-    const int lane = threadIdx.x & 31;
-    const int slice = blockIdx.x * kSellWarps + (threadIdx.x >> 5);
-    unsigned long long amb = 0ull, rsb = 0ull;
-    if (slice < s.nslices) {
-        const int row = s.sell_row[slice * 32 + lane];
-        const int64_t o0 = s.sell_off[slice] + lane, o1 = s.sell_off[slice + 1];
+    __shared__ double s_carry[kSellWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const SellSeg g = sell_seg<SEG>(s, wid, lane);
+    const int64_t o0 = g.o0, o1 = g.o1;
+    unsigned long long amb = 0ull;
+    double rsum = 0.0;
+    if (g.slice >= 0) {
+        const int row = s.sell_row[g.slice * 32 + lane];
         const int ei = row >= 0 ? exp_of_pow2(d[row]) : 0;
-        double rsum = 0.0;
         for (int64_t ob = o0; ob < o1; ob += 32 * kSellChunk) {
             double k[kSellChunk];
             int c[kSellChunk];
@@ -280,19 +355,31 @@ __global__ void __launch_bounds__(256) scale_sell_kernel(DevSched s, DevNum<T> n
                             ab | ((unsigned long long)__double_as_longlong(k[u]) & 0x8000000000000000ull);
                         out = (T)__longlong_as_double((long long)sb);     // d_i k d_j, exact
                         amb = ab > amb ? ab : amb;
-                        rsum += fabs(k[u]);
+                        if (!SEG) rsum += fabs(k[u]);
                     }
                     nm.sv[o] = out;
                 }
             }
         }
-        rsb = abs_bits(rsum);
     }
+    // ||K||_inf of a segmented row (the values again, from L1): a padding slot
+    // adds +0, which changes no sum of absolute values
+    if (SEG)
+        rsum = sell_sum<SEG>(g, wid, lane, s_carry, [&](double& acc) {
+            for (int64_t ob = o0; ob < o1; ob += 32 * kSellChunk) {
+                double k[kSellChunk];
+#pragma unroll
+                for (int u = 0; u < kSellChunk; ++u) k[u] = ob + 32 * u < o1 ? nm.kcopy[ob + 32 * u] : 0.0;
+#pragma unroll
+                for (int u = 0; u < kSellChunk; ++u)
+                    if (ob + 32 * u < o1) acc += fabs(k[u]);
+            }
+        });
+    unsigned long long rsb = g.last() ? abs_bits(rsum) : 0ull;
     // maxima of non-negative doubles as maxima of their bit patterns (integer shuffles)
     amb = warp_umax(amb);
     rsb = warp_umax(rsb);
     __shared__ unsigned long long s_am[kSellWarps], s_rs[kSellWarps];
-    const int wid = threadIdx.x >> 5;
     if (lane == 0) { s_am[wid] = amb; s_rs[wid] = rsb; }
     __syncthreads();
     // one atomic per block and quantity (per-row atomics serialise on one address)
@@ -304,28 +391,60 @@ __global__ void __launch_bounds__(256) scale_sell_kernel(DevSched s, DevNum<T> n
     }
 }
 
-// sum_k kv[o_k] x[c_k] over the slots of one lane's row, in slot (= CSR) order
-__device__ __forceinline__ double sell_row_dot(const DevSched& s, const double* __restrict__ kv,
-                                               const double* __restrict__ x, int64_t o0, int64_t o1)
+// sum_k kv[o_k] x[c_k] over each lane's row, in slot (= CSR) order; every
+// thread of the block calls it, the last segment's warp has the sum.
+template <bool SEG>
+__device__ __forceinline__ double sell_row_dot(const DevSched& s, const SellSeg& g, int wid, int lane,
+                                               double (*carry)[32], const double* __restrict__ kv,
+                                               const double* __restrict__ x)
 {
-    double acc = 0.0;
-    for (int64_t ob = o0; ob < o1; ob += 32 * kSellChunk) {
-        double k[kSellChunk];
-        int c[kSellChunk];
+    if (!SEG) {                                                    // throughput: few registers, many warps
+        double acc = 0.0;
+        for (int64_t ob = g.o0; ob < g.o1; ob += 32 * kSellChunk) {
+            double k[kSellChunk], xv[kSellChunk];
+            int c[kSellChunk];
 #pragma unroll
-        for (int u = 0; u < kSellChunk; ++u) {
-            const int64_t o = ob + 32 * u;
-            c[u] = o < o1 ? s.sell_ci[o] : -1;
-            k[u] = o < o1 ? kv[o] : 0.0;
+            for (int u = 0; u < kSellChunk; ++u) {
+                const int64_t o = ob + 32 * u;
+                c[u] = o < g.o1 ? s.sell_ci[o] : -1;
+                k[u] = o < g.o1 ? kv[o] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kSellChunk; ++u)
+                if (c[u] >= 0) acc = fma(k[u], xv[u], acc);
         }
-        double xv[kSellChunk];
+        return acc;
+    }
+    double k[kSellChunk], xv[kSellChunk];
+    int c[kSellChunk];
 #pragma unroll
-        for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : 0.0;
+    for (int u = 0; u < kSellChunk; ++u) {
+        const int64_t o = g.o0 + 32 * u;
+        c[u] = o < g.o1 ? s.sell_ci[o] : -1;
+        k[u] = o < g.o1 ? kv[o] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : 0.0;
+    return sell_sum<SEG>(g, wid, lane, carry, [&](double& acc) {
 #pragma unroll
         for (int u = 0; u < kSellChunk; ++u)
             if (c[u] >= 0) acc = fma(k[u], xv[u], acc);
-    }
-    return acc;
+        for (int64_t ob = g.o0 + 32 * kSellChunk; ob < g.o1; ob += 32 * kSellChunk) {
+#pragma unroll
+            for (int u = 0; u < kSellChunk; ++u) {
+                const int64_t o = ob + 32 * u;
+                c[u] = o < g.o1 ? s.sell_ci[o] : -1;
+                k[u] = o < g.o1 ? kv[o] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kSellChunk; ++u)
+                if (c[u] >= 0) acc = fma(k[u], xv[u], acc);
+        }
+    });
 }
 
 // ---------------------------------------------------------- front kernels
@@ -1268,15 +1387,16 @@ __global__ void __launch_bounds__(128) solve_bwd_cta_kernel(DevSched s, DevNum<T
 
 // y = b - K x (b != nullptr) or y = K x on the sliced copy of K, a lane per
 // row summing its entries in CSR order.
+template <bool SEG>
 __global__ void __launch_bounds__(256) spmv_sell_kernel(DevSched s, const double* __restrict__ kv,
                                                         const double* __restrict__ x, const double* __restrict__ b,
                                                         double* __restrict__ y)
 {
-    const int lane = threadIdx.x & 31;
-    const int slice = blockIdx.x * kSellWarps + (threadIdx.x >> 5);
-    if (slice >= s.nslices) return;
-    const int row = s.sell_row[slice * 32 + lane];
-    const double acc = sell_row_dot(s, kv, x, s.sell_off[slice] + lane, s.sell_off[slice + 1]);
+    __shared__ double s_carry[kSellWarps][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const SellSeg g = sell_seg<SEG>(s, wid, lane);
+    const int row = g.last() ? s.sell_row[g.slice * 32 + lane] : -1;
+    const double acc = sell_row_dot<SEG>(s, g, wid, lane, s_carry, kv, x);
     if (row >= 0) y[row] = b ? b[row] - acc : acc;
 }
 
@@ -1449,22 +1569,23 @@ cudaError_t launch_zero_stat(DevStat* stat, cudaStream_t st)
     return cudaMemsetAsync(stat, 0, sizeof(DevStat), st);
 }
 
-static inline int sell_blocks(const DevSched& s) { return cdiv(s.nslices, kSellWarps); }
+static inline int sell_blocks(const DevSched& s) { return s.sell_nblk ? s.sell_nblk : cdiv(s.nslices, kSellWarps); }
 
 cudaError_t launch_ruiz(const DevSched& s, const double* vals, int64_t bs_nnz, double* kcopy, unsigned short* keys,
                         int64_t bs_slot, double* d, double* dtmp, int iters, DevStat* stat, double** d_final,
                         int batch, cudaStream_t st)
 {
     const dim3 grid(sell_blocks(s), batch);
+    const auto kernel = s.sell_nblk ? ruiz_sell_kernel<true> : ruiz_sell_kernel<false>;
     double* a = d;
     double* b = dtmp;
     if (iters == 0) {
-        ruiz_sell_kernel<<<grid, 256, 0, st>>>(s, vals, bs_nnz, kcopy, keys, bs_slot, a, b, stat, 0, 1);
+        kernel<<<grid, 256, 0, st>>>(s, vals, bs_nnz, kcopy, keys, bs_slot, a, b, stat, 0, 1);
         *d_final = a;
         return cudaGetLastError();
     }
     for (int it = 0; it < iters; ++it) {
-        ruiz_sell_kernel<<<grid, 256, 0, st>>>(s, vals, bs_nnz, kcopy, keys, bs_slot, a, b, stat, it, 0);
+        kernel<<<grid, 256, 0, st>>>(s, vals, bs_nnz, kcopy, keys, bs_slot, a, b, stat, it, 0);
         double* t = a; a = b; b = t;
     }
     *d_final = a;
@@ -1475,7 +1596,8 @@ template <typename T>
 cudaError_t launch_scale(const DevSched& s, const DevNum<T>& nm, const double* d, int batch, cudaStream_t st)
 {
     (void)d;
-    scale_sell_kernel<T><<<dim3(sell_blocks(s), batch), 256, 0, st>>>(s, nm);
+    const auto kernel = s.sell_nblk ? scale_sell_kernel<T, true> : scale_sell_kernel<T, false>;
+    kernel<<<dim3(sell_blocks(s), batch), 256, 0, st>>>(s, nm);
     return cudaGetLastError();
 }
 
@@ -1607,13 +1729,13 @@ cudaError_t launch_solve_bwd_cta(const DevSched& s, const DevNum<T>& nm, const i
 cudaError_t launch_spmv_resid(const DevSched& s, const double* kv, const double* x, const double* b, double* r,
                               cudaStream_t st)
 {
-    spmv_sell_kernel<<<sell_blocks(s), 256, 0, st>>>(s, kv, x, b, r);
+    (s.sell_nblk ? spmv_sell_kernel<true> : spmv_sell_kernel<false>)<<<sell_blocks(s), 256, 0, st>>>(s, kv, x, b, r);
     return cudaGetLastError();
 }
 
 cudaError_t launch_spmv(const DevSched& s, const double* kv, const double* x, double* y, cudaStream_t st)
 {
-    spmv_sell_kernel<<<sell_blocks(s), 256, 0, st>>>(s, kv, x, nullptr, y);
+    (s.sell_nblk ? spmv_sell_kernel<true> : spmv_sell_kernel<false>)<<<sell_blocks(s), 256, 0, st>>>(s, kv, x, nullptr, y);
     return cudaGetLastError();
 }
 
@@ -1681,6 +1803,7 @@ cudaError_t launch_norms(int n, const double* a, double* out, cudaStream_t st)
 // omega); ||K||_inf comes from the refactorization's statistics. Each block
 // stores max |r|, |x|, |b| of its rows (as bits) in its slot of `part`;
 // omega_final_batched reduces the slots.
+template <bool SEG>
 __global__ void __launch_bounds__(256) resid_omega_part_kernel(DevSched s, const double* __restrict__ kv,
                                                                int64_t bs_slot, const double* __restrict__ x,
                                                                const double* __restrict__ b, double* __restrict__ r,
@@ -1693,19 +1816,19 @@ __global__ void __launch_bounds__(256) resid_omega_part_kernel(DevSched s, const
     x += (int64_t)inst * n;
     b += (int64_t)inst * n;
     r += (int64_t)inst * n;
+    __shared__ double s_carry[kSellWarps][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int slice = blockIdx.x * kSellWarps + wid;
+    const SellSeg g = sell_seg<SEG>(s, wid, lane);
+    const int row = g.last() ? s.sell_row[g.slice * 32 + lane] : -1;
     unsigned long long mr = 0ull, mx = 0ull, mb = 0ull;
-    if (slice < s.nslices) {
-        const int row = s.sell_row[slice * 32 + lane];
-        const double acc = sell_row_dot(s, kv, x, s.sell_off[slice] + lane, s.sell_off[slice + 1]);
-        if (row >= 0) {
-            const double ri = b[row] - acc;
-            r[row] = ri;
-            mr = abs_bits(ri);
-            mx = abs_bits(x[row]);
-            mb = abs_bits(b[row]);
-        }
+    const double acc = sell_row_dot<SEG>(s, g, wid, lane, s_carry, kv, x);
+    if (row >= 0) {
+        const double bi = b[row], xi = x[row];
+        const double ri = bi - acc;
+        r[row] = ri;
+        mr = abs_bits(ri);
+        mx = abs_bits(xi);
+        mb = abs_bits(bi);
     }
     mr = warp_umax(mr); mx = warp_umax(mx); mb = warp_umax(mb);
     if (lane == 0) { red[0][wid] = mr; red[1][wid] = mx; red[2][wid] = mb; }
@@ -1755,7 +1878,8 @@ cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t b
 {
     const int nblk = sell_blocks(s);
     unsigned long long* up = reinterpret_cast<unsigned long long*>(part);
-    resid_omega_part_kernel<<<dim3(nblk, batch), 256, 0, st>>>(s, kvals, bs_slot, x, b, r, up);
+    const auto kernel = s.sell_nblk ? resid_omega_part_kernel<true> : resid_omega_part_kernel<false>;
+    kernel<<<dim3(nblk, batch), 256, 0, st>>>(s, kvals, bs_slot, x, b, r, up);
     omega_final_batched_kernel<<<batch, 256, 0, st>>>(nblk, up, stat, omega);
     return cudaGetLastError();
 }

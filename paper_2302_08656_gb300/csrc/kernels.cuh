@@ -38,6 +38,8 @@ struct DevSched {
     const int* sell_row = nullptr;        // nslices * 32 (-1: no row)
     const int* sell_ci = nullptr;         // slots (-1: padding)
     const int* sell_src = nullptr;        // slots: CSR position (-1: padding)
+    const int4* sell_task = nullptr;      // work of each warp, kSellWarps per block (SellPlan::task)
+    int sell_nblk = 0;                    // ... and its blocks; 0: a warp takes a whole slice
 };
 
 // Device-side counters of one context, cleared at the start of each refactor.
@@ -347,7 +349,7 @@ template <typename T>
 cudaError_t launch_solve_post(const DevSched& s, const DevNum<T>& nm, double* x, int batch, cudaStream_t st);
 // per instance: r = b - K x, omega = ||r||_inf / (||K||_inf ||x||_inf + ||b||_inf) into omega[b],
 // K the sliced copy (instance stride bs_slot); part holds batch * resid_blocks(n) * 4 doubles
-constexpr int kResidRows = 64;         // rows per block of the partial-maxima buffer (an upper bound)
+constexpr int kResidRows = 32;         // a block has at least one slice of 32 rows (bounds the partial-maxima buffer)
 inline int resid_blocks(int n) { return (n + kResidRows - 1) / kResidRows; }
 // ||K||_inf of every instance is read from stat[inst].knorm_bits (the refactorization's scaling pass)
 cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t bs_slot, const double* x,

@@ -1176,7 +1176,8 @@ static int64_t plan_bytes(const Analysis& an, int n, int64_t nnz, const kkt_opti
     add((kCtrHead + 2 * B * nq) * 4); add((kCtrHead + 2 * B * nq) * 4); add(2 * 4);
     add((n + 1) * 4); add(std::max<int64_t>((int64_t)an.rel.size(), 1) * 4);
     add((3 * (int64_t)n + std::max<int64_t>((int64_t)an.rel.size(), 1)) * es);
-    add(((int64_t)sp.nslices + 1) * 8); add((int64_t)sp.nslices * 32 * 4); add(sp.slots * 4); add(sp.slots * 4);
+    add(((int64_t)sp.nslices + 1) * 8); add((int64_t)sp.nslices * 32 * 4); add((int64_t)sp.nblocks * kSellWarps * 16);
+    add(sp.slots * 4); add(sp.slots * 4);
     add(B * sp.slots * 2);
     return b;
 }
@@ -1206,6 +1207,7 @@ kkt_status kkt_plan(int32_t n, const int32_t* h_rowptr, const int32_t* h_colidx,
                      f12_total);
         SellPlan sp;
         build_sell(n, h_rowptr, h_colidx, kSellWindow, sp);
+        if (sp.nslices <= kSellSegmentWarps) segment_sell(sp);
         std::memset(out, 0, sizeof(*out));
         out->n = n;
         out->nnz = an.nnz;
@@ -1299,6 +1301,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
                      c->max_panel_global, inv_off, inv, f12_off, f12_total);
         // K's per-refactor copies live in the sliced layout: the assembly reads them at slots
         build_sell(n, h_rowptr, h_colidx, kSellWindow, sp);
+        if ((int64_t)sp.nslices * batch <= kSellSegmentWarps) segment_sell(sp);
         asm_src_sell.resize(c->an.asm_src.size());
         for (size_t e = 0; e < asm_src_sell.size(); ++e) asm_src_sell[e] = sp.csr2sell[c->an.asm_src[e]];
     } catch (...) {
@@ -1394,6 +1397,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     c->jac_buf = P.take<char>((3 * (size_t)n + std::max<size_t>(an.rel.size(), 1)) * es);
     int64_t* sell_off = P.take<int64_t>(sp.nslices + 1);
     int* sell_row = P.take<int>((int64_t)sp.nslices * 32);
+    int4* sell_task = P.take<int4>((int64_t)sp.nblocks * kSellWarps);
     int* sell_ci = P.take<int>(slots);
     int* sell_src = P.take<int>(slots);
     unsigned short* keys = P.take<unsigned short>(B * slots);
@@ -1440,6 +1444,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     e = e ? e : up(sell_off, sp.off.data(), (sp.nslices + 1) * 8);
     e = e ? e : up(sell_row, sp.row.data(), (size_t)sp.nslices * 32 * 4);
     e = e ? e : up(sell_ci, sp.ci.data(), slots * 4);
+    e = e ? e : up(sell_task, sp.task.data(), sp.task.size() * 4);
     e = e ? e : up(sell_src, sp.src.data(), slots * 4);
     e = e ? e : up(rel_ptr, an.rel_ptr.data(), (an.ns + 1) * 8);
     e = e ? e : up(rel, an.rel.data(), an.rel.size() * 4);
@@ -1496,6 +1501,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     s.rel_ptr = rel_ptr; s.rel = rel; s.panel_off = panel_off; s.cb_off = cb_off;
     s.cb_split = cb_split; s.inv_off = inv_off_d; s.inv = inv_d; s.f12_off = f12_off_d;
     s.nslices = sp.nslices; s.slots = slots;
+    s.sell_task = sell_task; s.sell_nblk = sp.nblocks;
     s.sell_off = sell_off; s.sell_row = sell_row; s.sell_ci = sell_ci; s.sell_src = sell_src;
     c->tsched = tp.ts;
     c->tsched.fr = tfr; c->tsched.kid = tkid; c->tsched.unit = tunit; c->tsched.inv = tinv;
