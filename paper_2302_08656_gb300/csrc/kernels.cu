@@ -1842,7 +1842,8 @@ __global__ void __launch_bounds__(256) resid_omega_part_kernel(DevSched s, const
 
 __global__ void __launch_bounds__(256) omega_final_batched_kernel(int nblk, const unsigned long long* __restrict__ part,
                                                                   const DevStat* __restrict__ stat,
-                                                                  double* __restrict__ omega)
+                                                                  double* __restrict__ omega,
+                                                                  double* __restrict__ maxima)
 {
     __shared__ unsigned long long red[3][8];
     const int inst = blockIdx.x;
@@ -1867,6 +1868,12 @@ __global__ void __launch_bounds__(256) omega_final_batched_kernel(int nblk, cons
         const double xmax = __longlong_as_double((long long)red[1][0]);
         const double bmax = __longlong_as_double((long long)red[2][0]);
         const double knorm = __longlong_as_double((long long)stat[inst].knorm_bits);
+        if (maxima) {
+            maxima[4 * inst] = rmax;
+            maxima[4 * inst + 1] = xmax;
+            maxima[4 * inst + 2] = bmax;
+            maxima[4 * inst + 3] = knorm;
+        }
         const double den = knorm * xmax + bmax;
         omega[inst] = den > 0.0 ? rmax / den : (den == 0.0 ? rmax : den);   // NaN stays NaN
     }
@@ -1874,13 +1881,13 @@ __global__ void __launch_bounds__(256) omega_final_batched_kernel(int nblk, cons
 
 cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t bs_slot, const double* x,
                                const double* b, double* r, double* part, const DevStat* stat, double* omega,
-                               int batch, cudaStream_t st)
+                               int batch, cudaStream_t st, double* maxima)
 {
     const int nblk = sell_blocks(s);
     unsigned long long* up = reinterpret_cast<unsigned long long*>(part);
     const auto kernel = s.sell_nblk ? resid_omega_part_kernel<true> : resid_omega_part_kernel<false>;
     kernel<<<dim3(nblk, batch), 256, 0, st>>>(s, kvals, bs_slot, x, b, r, up);
-    omega_final_batched_kernel<<<batch, 256, 0, st>>>(nblk, up, stat, omega);
+    omega_final_batched_kernel<<<batch, 256, 0, st>>>(nblk, up, stat, omega, maxima);
     return cudaGetLastError();
 }
 

@@ -351,10 +351,11 @@ cudaError_t launch_solve_post(const DevSched& s, const DevNum<T>& nm, double* x,
 // K the sliced copy (instance stride bs_slot); part holds batch * resid_blocks(n) * 4 doubles
 constexpr int kResidRows = 32;         // a block has at least one slice of 32 rows (bounds the partial-maxima buffer)
 inline int resid_blocks(int n) { return (n + kResidRows - 1) / kResidRows; }
-// ||K||_inf of every instance is read from stat[inst].knorm_bits (the refactorization's scaling pass)
+// ||K||_inf of every instance is read from stat[inst].knorm_bits (the refactorization's scaling pass);
+// maxima (optional): ||r||, ||x||, ||b||, ||K|| of each instance
 cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t bs_slot, const double* x,
                                const double* b, double* r, double* part, const DevStat* stat, double* omega,
-                               int batch, cudaStream_t st);
+                               int batch, cudaStream_t st, double* maxima = nullptr);
 
 // FP64 vector kernels for the residual and FGMRES (kv: one instance's sliced copy of K).
 cudaError_t launch_spmv_resid(const DevSched& s, const double* kv, const double* x, const double* b, double* r,
