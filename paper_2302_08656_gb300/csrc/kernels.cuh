@@ -260,6 +260,7 @@ struct TreeSched {
     // 1: every mini front has at most 32 rows, and the fused mode runs the forward step inside the
     // units (ti, 0) (a lane per row) in the plain unit order; 0: it runs the forward units of unit_fused
     int fwd_in = 0;
+    int cb32 = 0;                      // 1: 32-bit offsets reach every contribution block of an instance
     size_t kid_off = 0;                // shared-memory offset of the children's descriptors (factor kernel)
     const int* inv = nullptr;          // gather maps: parent CB row -> child CB row or -1
     // shared-memory layout parameters (host computed)

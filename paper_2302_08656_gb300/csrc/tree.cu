@@ -154,7 +154,7 @@ __device__ __forceinline__ bool panel_f32(const float* M, int Fr, int p0, int pk
     for (int k = 0; k < 8; ++k) a[k] = ((FULL || k < pk) && row < Fr) ? M[row + (p0 + k) * Fr] : 0.0f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const bool act = FULL || k < pk;                           // warp-uniform
+        if (!FULL && k >= pk) break;                               // warp-uniform
         float u[8];
 #pragma unroll
         for (int kk = k + 1; kk < 8; ++kk) u[kk] = __shfl_sync(0xffffffffu, a[kk], k);   // pivot row p0 + k
@@ -164,15 +164,13 @@ __device__ __forceinline__ bool panel_f32(const float* M, int Fr, int p0, int pk
         float r;
         if (FAST) {
             r = pivot_rcp_fast(piv);
-            ok = ok && (!act || pivot_rcp_fast_ok(piv));
+            ok = ok && pivot_rcp_fast_ok(piv);
         } else {
             r = pivot_rcp(piv);
         }
-        if (act) {
-            bad |= (int)b1;
-            pert += (int)p1;
-        }
-        const bool lk = act && tx == k, below = act && tx > k;
+        bad |= (int)b1;
+        pert += (int)p1;
+        const bool lk = tx == k, below = tx > k;
         a[k] = lk ? piv : (below ? a[k] * r : a[k]);               // l below the pivot
 #pragma unroll
         for (int kk = k + 1; kk < 8; ++kk)
@@ -218,7 +216,8 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
         for (int c = 0; c < 3; ++c) v[c] = (row < Fr && jb + 8 * c < Fc) ? M[row + (jb + 8 * c) * Fr] : 0.0f;
 #pragma unroll
         for (int k = 0; k < kPanel; ++k) {
-            const bool upd = (FULL || k < pk) && tx > k;
+            if (!FULL && k >= pk) break;                           // warp-uniform
+            const bool upd = tx > k;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const float u = __shfl_sync(0xffffffffu, v[c], k);   // row p0 + k: final at step k
@@ -363,6 +362,38 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         const bool fwd_here = !MULTI && fused == kFwdInside && ut.tj == 0;   // warp 0's forward step below
         T xf = T(0);
         if (fwd_here && tid < w) xf = nm.vin[d.first + tid];       // w <= 32; vin: the lead unit overwrites vec
+        // where a thread's first children's entries are (kAhead per column):
+        // found before the wait, so that the loads are issued right after it
+        // (with partial pivot panels of their own length, below: 70k buses
+        // FP32 step 1691 -> 1666 us, FP64 2891 -> 2793)
+        const bool ahead = ts.cb32 && Fr <= 32 && Fc <= 32 && nk <= 32;
+        constexpr int kAhead = 2;
+        constexpr unsigned kNone = 0xffffffffu;
+        T acc[4];
+        unsigned mk[4], off[kAhead][4];
+        if (ahead) {
+            __syncthreads();                                       // maps and original entries are in place
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = ty + 8 * k;
+                mk[k] = __ballot_sync(0xffffffffu, j < Fc && tx < nk && cmap[j * KP + tx] >= 0);
+                acc[k] = tx < Fr && j < Fc ? M[tx + j * Fr] : T(0);
+            }
+#pragma unroll
+            for (int g = 0; g < kAhead; ++g)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    off[g][k] = kNone;
+                    if (mk[k]) {
+                        const int c = __ffs(mk[k]) - 1;
+                        mk[k] &= mk[k] - 1u;
+                        const int sr = tx < Fr ? rmap[c * W + tx] : -1;
+                        if (sr >= 0)
+                            off[g][k] = (unsigned)kids[c].cb_off + (unsigned)sr +
+                                        (unsigned)cmap[(ty + 8 * k) * KP + c] * (unsigned)kids[c].mc;
+                    }
+                }
+        }
         // ---- wait for the children (bounded; lane l of warp 0 polls children l, l + 32)
         if (tid == 0) {
             s_ok = 1;
@@ -382,7 +413,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             break;
         }
         // ---- children's contributions, in child order for every entry; each
-        // thread holds four entries of one row and keeps up to 16 loads in
+        // thread holds four entries of one row and keeps up to 8 loads in
         // flight. A warp visits, column by column, only the children that
         // reach the column (a ballot over the children): fronts of the lower
         // tree levels have up to 37 children of a few rows each, and testing
@@ -393,20 +424,32 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             for (int jb = ty; jb < Fc; jb += 32) {
                 const int i = ib + tx;
                 const bool in = i < Fr;
-                T acc[4];
+                if (ahead) {
+                    T v[kAhead][4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = in && jb + 8 * k < Fc ? M[i + (jb + 8 * k) * Fr] : T(0);
+                    for (int g = 0; g < kAhead; ++g)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) v[g][k] = off[g][k] != kNone ? __ldcg(nm.cb + off[g][k]) : T(0);
+#pragma unroll
+                    for (int g = 0; g < kAhead; ++g)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (off[g][k] != kNone) acc[k] += v[g][k];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[k] = in && jb + 8 * k < Fc ? M[i + (jb + 8 * k) * Fr] : T(0);
+                }
                 for (int h = 0; h < nk; h += 32) {
-                    unsigned mk[4];                                // children h + bit that reach column jb + 8 k
+                    if (!ahead)                                    // children h + bit that reach column jb + 8 k
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mk[k] = __ballot_sync(0xffffffffu, jb + 8 * k < Fc && h + tx < nk &&
-                                                               cmap[(jb + 8 * k) * KP + h + tx] >= 0);
+                        for (int k = 0; k < 4; ++k)
+                            mk[k] = __ballot_sync(0xffffffffu, jb + 8 * k < Fc && h + tx < nk &&
+                                                                   cmap[(jb + 8 * k) * KP + h + tx] >= 0);
                     while (mk[0] | mk[1] | mk[2] | mk[3]) {
-                        T v[4][4];
+                        T v[2][4];
                         unsigned valid = 0u;
 #pragma unroll
-                        for (int g = 0; g < 4; ++g)
+                        for (int g = 0; g < 2; ++g)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 v[g][k] = T(0);
@@ -422,7 +465,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                                 }
                             }
 #pragma unroll
-                        for (int g = 0; g < 4; ++g)
+                        for (int g = 0; g < 2; ++g)
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
                                 if (valid & (1u << (4 * g + k))) acc[k] += v[g][k];
@@ -612,9 +655,9 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
 }
 
 // Entry points: in single precision the kernel is held to 64 registers, so
-// that 4 CTAs fit on an SM; double precision keeps the compiler's choice.
+// that 4 CTAs fit on an SM; in double precision to 80, for 3.
 template <typename T, bool MULTI>
-__global__ void __launch_bounds__(256) tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr,
+__global__ void __launch_bounds__(256, 3) tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr,
                                                           int* stall, long long limit, int fused, int u0, int nu,
                                                           int tick, const TreeJob<T>* jobs, const TreeSeg* segs,
                                                           int nseg)

@@ -141,6 +141,7 @@ void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
     ts.max_kids = std::max(ts.max_kids, 1);
     ts.kid_pitch = ts.max_kids | 1;
     ts.fwd_in = ts.map_w <= 32 ? 1 : 0;
+    ts.cb32 = an.cb_total < (int64_t)0xffffffffu ? 1 : 0;
     ts.fwd_stage = (size_t)ts.max_fw * es <= kStageLimit ? 1 : 0;
     ts.bwd_stage = 2 * (size_t)ts.max_wm * es <= kStageLimit ? 1 : 0;   // two fronts staged at a time
     // forward chains: the children's entries of the largest front's children
