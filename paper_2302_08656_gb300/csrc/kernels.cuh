@@ -121,10 +121,14 @@ __device__ __forceinline__ double pivot_rcp_fast(double d)
     const double e = fma(-d, x0, 1.0);
     return fma(x0, fma(e, e, e), x0);
 }
+// The division itself is a function of its own: inlined, the compiler puts its
+// six FP64 instructions in front of the range test (114 of the 630 cycles of a
+// pivot). It takes the fast value, which so is formed before the test.
+static __device__ __noinline__ double pivot_rcp_div(double d, double) { return 1.0 / d; }
 __device__ __forceinline__ double pivot_rcp(double d)
 {
-    if (!pivot_rcp_fast_ok(d)) return 1.0 / d;
-    return pivot_rcp_fast(d);
+    const double r = pivot_rcp_fast(d);
+    return pivot_rcp_fast_ok(d) ? r : pivot_rcp_div(d, r);
 }
 __device__ __forceinline__ bool pivot_rcp_fast_ok(float d)
 {

@@ -231,6 +231,15 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
     __syncthreads();
 }
 
+// A pivot of the double-precision elimination that is not simply kept with its
+// Newton reciprocal (r, unused: see pivot_rcp_div): static pivoting, then
+// pivot_rcp. Returns the pivot and its reciprocal; counts the event if count.
+__device__ __noinline__ double2 pivot_slow(double x, double, double floorT, DevStat* stat, bool count)
+{
+    const double pv = static_pivot(x, floorT, stat, count);
+    return make_double2(pv, pivot_rcp(pv));
+}
+
 // ------------------------------------------------------------- refactor
 
 // Unit (q, ti, tj) of instance b. Mini front M (Fr x Fc, column-major, ld Fr):
@@ -495,7 +504,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 if (tx == 0 && n_bad) atomicExch(&nm.stat->numeric_bad, 1);
                 if (tx == 0 && n_pert) atomicAdd(&nm.stat->n_perturbed, n_pert);
             }
-        } else if (Fr <= 32 && Fc <= 32) {
+        } else if (sizeof(T) == 8 && Fr <= 32 && Fc <= 32) {
             // mini fronts of at most 32 x 32 (always when w <= 16). GB300 runs
             // one FP64 warp instruction per ~64 cycles per sub-partition, masked
             // lanes included, so the elimination is bound by the FP64
@@ -506,15 +515,30 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             // columns each from p+2 (lane -> row), a warp whose columns are all
             // eliminated issues nothing, and warp 4, which shares a
             // sub-partition with warp 0, takes the last group.
+            // A pivot is computed by every lane of warp 0 from lane 0's entry
+            // (one lane alone: 46 cycles of divergence), and its reciprocal
+            // starts at once: that the entry is kept as it is and in the
+            // range of the Newton step is tested on its high word beside it
+            // (lo, hi), and pivot_slow repeats the rare others. A pivot's
+            // chain, update, reciprocal, scaling and exchanges, is 430 cycles
+            // so, 630 with the static pivot and the range test in it.
+            unsigned lo = (unsigned)__double2hiint((double)floorT) + 1u;   // above it: not below the floor
+            lo = lo > (23u << 20) ? lo : 23u << 20;                // pivot_rcp_fast_ok: biased exponents 23 .. 2023
+            const unsigned hi = (2023u << 20) | 0xfffffu;
+            auto pivot = [&](double x, double& r) {
+                r = pivot_rcp_fast(x);
+                const unsigned ax = (unsigned)__double2hiint(x) & 0x7fffffffu;
+                if (ax >= lo && ax <= hi) return x;                // warp-uniform
+                const double2 q = pivot_slow(x, r, (double)floorT, nm.stat, lead && tx == 0);
+                r = q.y;
+                return q.x;
+            };
             if (ty == 0 && w > 0) {
-                T r = T(0);
-                if (tx == 0) {
-                    const T pv = static_pivot(M[0], floorT, nm.stat, lead);
-                    M[0] = pv;
-                    r = pivot_rcp(pv);
-                }
-                r = __shfl_sync(0xffffffffu, r, 0);
-                if (1 + tx < Fr) M[1 + tx] *= r;
+                double r;
+                const T pv = (T)pivot((double)M[0], r);
+                __syncwarp();
+                if (tx == 0) M[0] = pv;
+                if (1 + tx < Fr) M[1 + tx] *= (T)r;
             }
             __syncthreads();
             const int g = ty < 4 ? ty - 1 : (ty == 4 ? 6 : ty - 2);
@@ -530,13 +554,9 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                         mv -= l * M[p + j * Fr];
                     }
                     if (p + 1 < w) {                               // warp-uniform
-                        T r = T(0);
-                        if (tx == 0) {
-                            mv = static_pivot(mv, floorT, nm.stat, lead);
-                            r = pivot_rcp(mv);
-                        }
-                        r = __shfl_sync(0xffffffffu, r, 0);
-                        if (tx > 0) mv *= r;
+                        double r;
+                        const T pv = (T)pivot((double)__shfl_sync(0xffffffffu, mv, 0), r);
+                        mv = tx == 0 ? pv : mv * (T)r;
                     }
                     if (act) M[i + j * Fr] = mv;
                 } else {
