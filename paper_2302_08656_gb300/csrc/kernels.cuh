@@ -404,7 +404,7 @@ cudaError_t launch_tree_factor_group(const TreeJob<T>* jobs, const TreeSeg* segs
 template <typename T>
 cudaError_t launch_tree_factor(const DevSched& s, const TreeSched& t, const DevNum<T>& nm, int batch, int* ctr,
                                int* stall, long long spin_limit, int grid, size_t smem, int fused, int u0, int nu,
-                               int tick, cudaStream_t st);
+                               int tick, bool narrow, cudaStream_t st);
 template <typename T>
 cudaError_t launch_tree_fwd(const DevSched& s, const TreeSched& t, const DevNum<T>& nm, int batch, int* ctr,
                             long long spin_limit, int grid, size_t smem, cudaStream_t st);

@@ -552,12 +552,12 @@ kkt_status factor_levels(kkt_ctx* c, DevNum<T>& nm, cudaStream_t st, bool fused 
         if (us > 0) {
             Launch L(c, st, KK_TREE_FACTOR, 1);
             KKT_CUDA(launch_tree_factor<T>(c->sched, c->tsched, nm, B, c->ctr_fac, c->stall, c->opt.spin_limit,
-                                           c->tf_grid, c->tf_smem, mode, 0, us, 0, st));
+                                           c->tf_grid, c->tf_smem, mode, 0, us, 0, false, st));
         }
         if (us < nu) {
             Launch L(c, st, KK_TREE_FACTOR, 1);
             KKT_CUDA(launch_tree_factor<T>(c->sched, c->tsched, nm, B, c->ctr_fac, c->stall, c->opt.spin_limit,
-                                           c->tf_grid_narrow, c->tf_smem, mode, us, nu - us, 3, st));
+                                           c->tf_grid_narrow, c->tf_smem, mode, us, nu - us, 3, true, st));
         }
     }
     return KKT_OK;

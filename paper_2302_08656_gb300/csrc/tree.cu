@@ -180,14 +180,14 @@ __device__ __forceinline__ bool panel_f32(const float* M, int Fr, int p0, int pk
 }
 
 // One kPanel = 8 step of the single-precision elimination of a mini front M
-// (Fr x Fc <= 32 x 32, ld Fr) by 256 threads (32 x 8: lane -> row, warp ->
-// column group): warp 0 factors the panel (pivot columns p0 .. p0 + pk - 1,
+// (Fr x Fc <= 32 x 32, ld Fr) by NW warps (lane -> row, warp -> column
+// group): warp 0 factors the panel (pivot columns p0 .. p0 + pk - 1,
 // lane -> row p0 + lane) in registers without a CTA barrier; then every warp
-// applies it to its trailing columns j = p0 + pk + warp + 8 c (lane -> row,
+// applies it to its trailing columns j = p0 + pk + warp + NW c (lane -> row,
 // one shuffle per pivot for the row's U entry, its three columns
 // interleaved). Each entry still receives its updates in pivot order with
 // the same roundings as the one-pivot schedule. FULL: pk = 8.
-template <bool FULL>
+template <bool FULL, int NW>
 __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, int pk, float floorT, int& n_bad,
                                               int& n_pert)
 {
@@ -210,10 +210,10 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
     float lp[kPanel];
 #pragma unroll
     for (int k = 0; k < kPanel; ++k) lp[k] = ((FULL || k < pk) && row < Fr) ? M[row + (p0 + k) * Fr] : 0.0f;
-    for (int jb = p0 + pk + ty; jb < Fc; jb += 24) {
+    for (int jb = p0 + pk + ty; jb < Fc; jb += 3 * NW) {
         float v[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] = (row < Fr && jb + 8 * c < Fc) ? M[row + (jb + 8 * c) * Fr] : 0.0f;
+        for (int c = 0; c < 3; ++c) v[c] = (row < Fr && jb + NW * c < Fc) ? M[row + (jb + NW * c) * Fr] : 0.0f;
 #pragma unroll
         for (int k = 0; k < kPanel; ++k) {
             if (!FULL && k >= pk) break;                           // warp-uniform
@@ -226,7 +226,7 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            if (row < Fr && jb + 8 * c < Fc) M[row + (jb + 8 * c) * Fr] = v[c];
+            if (row < Fr && jb + NW * c < Fc) M[row + (jb + NW * c) * Fr] = v[c];
     }
     __syncthreads();
 }
@@ -257,11 +257,12 @@ __device__ __noinline__ double2 pivot_slow(double x, double, double floorT, DevS
 // Tickets and the abort flag come from the group's counter block (ctr);
 // completion counters are each context's own. The descriptors of the current
 // unit's context are cached in shared memory.
-template <typename T, bool MULTI>
+template <typename T, bool MULTI, int NT>
 __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, DevNum<T> nm0_p, int B_p, int* ctr,
                                                  int* stall, long long limit, int fused, int u0, int nu, int tick,
                                                  const TreeJob<T>* jobs, const TreeSeg* segs, int nseg)
 {
+    constexpr int NW = NT / 32, KC = 32 / NW;                  // warps; columns of a thread
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ TreeUnit su;                                    // the current unit and its front
     TreeFront& d = su.d;
@@ -291,7 +292,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             }
             __syncthreads();
             if (s_switch) {
-                copy_words(reinterpret_cast<TreeJob<T>*>(sj_raw), jobs + s_job, 1, tid, 256);
+                copy_words(reinterpret_cast<TreeJob<T>*>(sj_raw), jobs + s_job, 1, tid, NT);
                 __syncthreads();
             }
             const TreeSeg sg = segs[s_seg];
@@ -320,13 +321,13 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         int* rmap = reinterpret_cast<int*>(smraw + off_map);
         int* cmap = rmap + ts.max_kids * W;
         TreeKid* kids = reinterpret_cast<TreeKid*>(smraw + ts.kid_off);
-        copy_words(&su, units + (MULTI ? 0 : u0) + ul, 1, tid, 256);
+        copy_words(&su, units + (MULTI ? 0 : u0) + ul, 1, tid, NT);
         __syncthreads();
         const FrontTile ut = su.u;
         const int q = ut.front;
         const DevNum<T> nm = nm0.at(b);
         if (ut.ti < 0) {                                           // forward-solve unit (fused mode)
-            if (!fwd_unit<T, 256>(s, ts, nm, d, q, kids, s_cut, &s_ok, smraw, fwd_done + (int64_t)b * ts.nq,
+            if (!fwd_unit<T, NT>(s, ts, nm, d, q, kids, s_cut, &s_ok, smraw, fwd_done + (int64_t)b * ts.nq,
                                   done + (int64_t)b * ts.nq, ctr + 1, limit)) {
                 if (tid == 0) atomicExch(&nm.stat->timeout, 1);
                 break;
@@ -341,10 +342,10 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         const int nk = d.kid_end - d.kid_begin;
         const bool lead = ut.ti == 0 && ut.tj == 0;
         // ---- everything that does not depend on the children
-        for (int e = tid; e < Fr * Fc; e += 256) M[e] = T(0);
-        copy_words(kids, ts.kid + d.kid_begin, nk, tid, 256);
+        for (int e = tid; e < Fr * Fc; e += NT) M[e] = T(0);
+        copy_words(kids, ts.kid + d.kid_begin, nk, tid, NT);
         __syncthreads();
-        for (int c = ty; c < nk; c += 8) {                         // a warp per child
+        for (int c = ty; c < nk; c += NW) {                         // a warp per child
             const int* inv = ts.inv + d.inv_off + (int64_t)c * m - w;
             for (int i = tx; i < W; i += 32) {
                 if (i < Fr) rmap[c * W + i] = i >= w ? inv[i0 + i] : -1;
@@ -359,7 +360,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 cmap[r * KP + c] = tt;
             }
         }
-        for (int64_t e = d.asm_begin + tid; e < d.asm_end; e += 256) {
+        for (int64_t e = d.asm_begin + tid; e < d.asm_end; e += NT) {
             const int pos = s.asm_pos[e];
             const int bc = pos / F, a = pos - bc * F;
             const int lr = a < w ? a : ((unsigned)(a - w - i0) < (unsigned)nr ? a - i0 : -1);
@@ -378,20 +379,20 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         const bool ahead = ts.cb32 && Fr <= 32 && Fc <= 32 && nk <= 32;
         constexpr int kAhead = 2;
         constexpr unsigned kNone = 0xffffffffu;
-        T acc[4];
-        unsigned mk[4], off[kAhead][4];
+        T acc[KC];
+        unsigned mk[KC], off[kAhead][KC];
         if (ahead) {
             __syncthreads();                                       // maps and original entries are in place
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int j = ty + 8 * k;
+            for (int k = 0; k < KC; ++k) {
+                const int j = ty + NW * k;
                 mk[k] = __ballot_sync(0xffffffffu, j < Fc && tx < nk && cmap[j * KP + tx] >= 0);
                 acc[k] = tx < Fr && j < Fc ? M[tx + j * Fr] : T(0);
             }
 #pragma unroll
             for (int g = 0; g < kAhead; ++g)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < KC; ++k) {
                     off[g][k] = kNone;
                     if (mk[k]) {
                         const int c = __ffs(mk[k]) - 1;
@@ -399,7 +400,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                         const int sr = tx < Fr ? rmap[c * W + tx] : -1;
                         if (sr >= 0)
                             off[g][k] = (unsigned)kids[c].cb_off + (unsigned)sr +
-                                        (unsigned)cmap[(ty + 8 * k) * KP + c] * (unsigned)kids[c].mc;
+                                        (unsigned)cmap[(ty + NW * k) * KP + c] * (unsigned)kids[c].mc;
                     }
                 }
         }
@@ -422,7 +423,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             break;
         }
         // ---- children's contributions, in child order for every entry; each
-        // thread holds four entries of one row and keeps up to 8 loads in
+        // thread holds KC entries of one row and keeps up to 8 loads in
         // flight. A warp visits, column by column, only the children that
         // reach the column (a ballot over the children): fronts of the lower
         // tree levels have up to 37 children of a few rows each, and testing
@@ -434,55 +435,59 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 const int i = ib + tx;
                 const bool in = i < Fr;
                 if (ahead) {
-                    T v[kAhead][4];
+                    T v[kAhead][KC];
 #pragma unroll
                     for (int g = 0; g < kAhead; ++g)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) v[g][k] = off[g][k] != kNone ? __ldcg(nm.cb + off[g][k]) : T(0);
+                        for (int k = 0; k < KC; ++k) v[g][k] = off[g][k] != kNone ? __ldcg(nm.cb + off[g][k]) : T(0);
 #pragma unroll
                     for (int g = 0; g < kAhead; ++g)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
+                        for (int k = 0; k < KC; ++k)
                             if (off[g][k] != kNone) acc[k] += v[g][k];
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[k] = in && jb + 8 * k < Fc ? M[i + (jb + 8 * k) * Fr] : T(0);
+                    for (int k = 0; k < KC; ++k) acc[k] = in && jb + NW * k < Fc ? M[i + (jb + NW * k) * Fr] : T(0);
                 }
                 for (int h = 0; h < nk; h += 32) {
                     if (!ahead)                                    // children h + bit that reach column jb + 8 k
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            mk[k] = __ballot_sync(0xffffffffu, jb + 8 * k < Fc && h + tx < nk &&
-                                                                   cmap[(jb + 8 * k) * KP + h + tx] >= 0);
-                    while (mk[0] | mk[1] | mk[2] | mk[3]) {
-                        T v[2][4];
+                        for (int k = 0; k < KC; ++k)
+                            mk[k] = __ballot_sync(0xffffffffu, jb + NW * k < Fc && h + tx < nk &&
+                                                                   cmap[(jb + NW * k) * KP + h + tx] >= 0);
+                    for (;;) {
+                        unsigned any = 0u;
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) any |= mk[k];
+                        if (!any) break;
+                        T v[2][KC];
                         unsigned valid = 0u;
 #pragma unroll
                         for (int g = 0; g < 2; ++g)
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
+                            for (int k = 0; k < KC; ++k) {
                                 v[g][k] = T(0);
                                 if (mk[k]) {
                                     const int c = h + __ffs(mk[k]) - 1;
                                     mk[k] &= mk[k] - 1u;
                                     const int sr = in ? rmap[c * W + i] : -1;
-                                    const int sc = cmap[(jb + 8 * k) * KP + c];
+                                    const int sc = cmap[(jb + NW * k) * KP + c];
                                     if (sr >= 0) {
                                         v[g][k] = __ldcg(nm.cb + kids[c].cb_off + sr + (int64_t)sc * kids[c].mc);
-                                        valid |= 1u << (4 * g + k);
+                                        valid |= 1u << (KC * g + k);
                                     }
                                 }
                             }
 #pragma unroll
                         for (int g = 0; g < 2; ++g)
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                if (valid & (1u << (4 * g + k))) acc[k] += v[g][k];
+                            for (int k = 0; k < KC; ++k)
+                                if (valid & (1u << (KC * g + k))) acc[k] += v[g][k];
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (in && jb + 8 * k < Fc) M[i + (jb + 8 * k) * Fr] = acc[k];
+                for (int k = 0; k < KC; ++k)
+                    if (in && jb + NW * k < Fc) M[i + (jb + NW * k) * Fr] = acc[k];
             }
         __syncthreads();
         // ---- w pivot steps of right-looking elimination without pivoting, one
@@ -496,9 +501,9 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             for (int p0 = 0; p0 < w; p0 += 8) {
                 const int pk = min(8, w - p0);
                 if (pk == 8)
-                    elim_step_f32<true>(Mf, Fr, Fc, p0, pk, fl, n_bad, n_pert);
+                    elim_step_f32<true, NW>(Mf, Fr, Fc, p0, pk, fl, n_bad, n_pert);
                 else
-                    elim_step_f32<false>(Mf, Fr, Fc, p0, pk, fl, n_bad, n_pert);
+                    elim_step_f32<false, NW>(Mf, Fr, Fc, p0, pk, fl, n_bad, n_pert);
             }
             if (ty == 0 && lead && (n_bad | n_pert)) {                 // warp-uniform
                 if (tx == 0 && n_bad) atomicExch(&nm.stat->numeric_bad, 1);
@@ -511,7 +516,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             // instructions issued. Warp 0 owns column p+1 only: at step p it
             // finishes the next pivot (lane 0), broadcasts its reciprocal and
             // stores column p+1 already scaled, so at step p+1 every other warp
-            // reads l_i,p+1 and issues FMAs alone. Warps 1-7 own five adjacent
+            // reads l_i,p+1 and issues FMAs alone. The other warps own CG adjacent
             // columns each from p+2 (lane -> row), a warp whose columns are all
             // eliminated issues nothing, and warp 4, which shares a
             // sub-partition with warp 0, takes the last group.
@@ -541,7 +546,9 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 if (1 + tx < Fr) M[1 + tx] *= (T)r;
             }
             __syncthreads();
-            const int g = ty < 4 ? ty - 1 : (ty == 4 ? 6 : ty - 2);
+            // group of warp ty: the last ones to the warps that share warp 0's sub-partition
+            constexpr int CG = NW == 8 ? 5 : 2;
+            const int g = ty & 3 ? ty / 4 * 3 + (ty & 3) - 1 : NW / 4 * 3 + ty / 4 - 1;
             for (int p = 0; p < w; ++p) {
                 const int i = p + 1 + tx;
                 if (ty == 0) {
@@ -560,20 +567,20 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                     }
                     if (act) M[i + j * Fr] = mv;
                 } else {
-                    const int jg = p + 2 + 5 * g;
+                    const int jg = p + 2 + CG * g;
                     if (jg < Fc && i < Fr) {
                         const T l = M[i + p * Fr];
-                        T mv[5], uv[5];
+                        T mv[CG], uv[CG];
 #pragma unroll
-                        for (int k = 0; k < 5; ++k) {
+                        for (int k = 0; k < CG; ++k) {
                             const int j = jg + k;
                             mv[k] = j < Fc ? M[i + j * Fr] : T(0);
                             uv[k] = j < Fc ? M[p + j * Fr] : T(0);
                         }
 #pragma unroll
-                        for (int k = 0; k < 5; ++k) mv[k] -= l * uv[k];
+                        for (int k = 0; k < CG; ++k) mv[k] -= l * uv[k];
 #pragma unroll
-                        for (int k = 0; k < 5; ++k) {
+                        for (int k = 0; k < CG; ++k) {
                             const int j = jg + k;
                             if (j < Fc) M[i + j * Fr] = mv[k];
                         }
@@ -590,11 +597,11 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             __syncthreads();
             for (int p = 0; p < w; ++p) {
                 const T rinv = s_rinv[p];
-                if (p > 0 && ty == (p - 1) % 8)                    // deferred scaling of column p-1
+                if (p > 0 && ty == (p - 1) % NW)                    // deferred scaling of column p-1
                     for (int i = p + tx; i < Fr; i += 32) M[i + (p - 1) * Fr] *= s_rinv[p - 1];
                 for (int i = p + 1 + tx; i < Fr; i += 32) {
                     const T l = M[i + p * Fr] * rinv;
-                    for (int j = p + 1 + ty; j < Fc; j += 8) {
+                    for (int j = p + 1 + ty; j < Fc; j += NW) {
                         const T a = M[i + j * Fr] - l * M[p + j * Fr];
                         if (i == p + 1 && j == p + 1 && p + 1 < w) {
                             const T pv = static_pivot(a, floorT, nm.stat, lead);
@@ -608,29 +615,29 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 __syncthreads();
             }
             if (w > 0)
-                for (int i = w + tid; i < Fr; i += 256) M[i + (w - 1) * Fr] *= s_rinv[w - 1];
+                for (int i = w + tid; i < Fr; i += NT) M[i + (w - 1) * Fr] *= s_rinv[w - 1];
             __syncthreads();
         }
         // ---- results: the CB tile, all that the parent's units wait for, first
-        // and signalled by warp 7 (the panel too where forward units read it);
+        // and signalled by the last warp (the panel too where forward units read it);
         // then pivot block (lead unit), L21 rows (tj == 0), U12 columns (ti == 0)
         T* C = nm.cb + d.cb_off;
-        for (int c = ty; c < nc; c += 8)
+        for (int c = ty; c < nc; c += NW)
             for (int r = tx; r < nr; r += 32) C[(i0 + r) + (int64_t)(j0 + c) * m] = M[(w + r) + (w + c) * Fr];
         if (fused != kFwdUnits) {
             __syncthreads();
-            if (tid == 224) red_release(done + (int64_t)b * ts.nq + q);
+            if (tid == NT - 32) red_release(done + (int64_t)b * ts.nq + q);
         }
         T* pan = nm.panel + d.panel_off;
         if (lead)
-            for (int c = ty; c < w; c += 8)
+            for (int c = ty; c < w; c += NW)
                 for (int a = tx; a < w; a += 32) pan[a + (int64_t)c * F] = M[a + c * Fr];
         if (ut.tj == 0)
-            for (int c = ty; c < w; c += 8)
+            for (int c = ty; c < w; c += NW)
                 for (int r = tx; r < nr; r += 32) pan[(w + i0 + r) + (int64_t)c * F] = M[(w + r) + c * Fr];
         if (ut.ti == 0) {
             T* U12 = pan + (int64_t)F * w;
-            for (int c = ty; c < nc; c += 8)
+            for (int c = ty; c < nc; c += NW)
                 for (int a = tx; a < w; a += 32) U12[a + (int64_t)(j0 + c) * w] = M[a + (w + c) * Fr];
         }
         if (fused == kFwdUnits) {
@@ -674,30 +681,24 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
     }
 }
 
-// Entry points: in single precision the kernel is held to 64 registers, so
-// that 4 CTAs fit on an SM; in double precision to 80, for 3.
-template <typename T, bool MULTI>
-__global__ void __launch_bounds__(256, 3) tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr,
-                                                          int* stall, long long limit, int fused, int u0, int nu,
-                                                          int tick, const TreeJob<T>* jobs, const TreeSeg* segs,
-                                                          int nseg)
+// Entry points, NT threads per CTA. kTreeNt on the wide levels: in single
+// precision held to 64 registers, so that 4 CTAs fit on an SM, in double
+// precision to 80, for 3. The narrow top of the tree, one CTA per SM, takes
+// kTreeNtNarrow threads: a warp starts one FP64 instruction per 64 cycles, so
+// with 7 warps and 5 columns each the trailing update of a pivot took 726
+// cycles against 520 of the pivot's own chain; 15 warps take 2 columns each, and
+// loads and gathers have twice the threads. refactor_refine 200 buses FP64 300
+// -> 283 us, 2,003 FP32 347 -> 329, 9,973 FP64 967 -> 943, 25,000 FP64 1331 ->
+// 1304, FP32 920 -> 883. (The wide levels with 128 threads, twice the CTAs: 70,000
+// buses FP32 1759 -> 1863, FP64 2957 -> 3149.)
+constexpr int kTreeNt = 256, kTreeNtNarrow = 512;
+template <typename T, bool MULTI, int NT>
+__global__ void __launch_bounds__(NT, NT == kTreeNtNarrow ? 1 : sizeof(T) == 4 ? 4 : 3)
+tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr, int* stall, long long limit, int fused,
+                   int u0, int nu, int tick, const TreeJob<T>* jobs, const TreeSeg* segs, int nseg)
 {
-    tree_factor_body<T, MULTI>(s, ts, nm, B, ctr, stall, limit, fused, u0, nu, tick, jobs, segs, nseg);
+    tree_factor_body<T, MULTI, NT>(s, ts, nm, B, ctr, stall, limit, fused, u0, nu, tick, jobs, segs, nseg);
 }
-
-template <bool MULTI>
-__global__ void __launch_bounds__(256, 4) tree_factor_kernel_f32(DevSched s, TreeSched ts, DevNum<float> nm, int B,
-                                                                 int* ctr, int* stall, long long limit, int fused,
-                                                                 int u0, int nu, int tick, const TreeJob<float>* jobs,
-                                                                 const TreeSeg* segs, int nseg)
-{
-    tree_factor_body<float, MULTI>(s, ts, nm, B, ctr, stall, limit, fused, u0, nu, tick, jobs, segs, nseg);
-}
-
-template <bool MULTI>
-auto tree_factor_entry(const float*) { return tree_factor_kernel_f32<MULTI>; }
-template <bool MULTI>
-auto tree_factor_entry(const double*) { return tree_factor_kernel<double, MULTI>; }
 
 // ------------------------------------------------------ forward substitution
 
@@ -1331,8 +1332,8 @@ cudaError_t tree_grid(int kind, size_t smem, int* grid)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
-    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_entry<false>((const T*)nullptr), 256, smem);
-    else if (kind == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_entry<true>((const T*)nullptr), 256, smem);
+    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_kernel<T, false, kTreeNt>, kTreeNt, smem);
+    else if (kind == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_kernel<T, true, kTreeNt>, kTreeNt, smem);
     else if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_fwd_kernel<T>, 128, smem);
     else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_bwd_kernel<T>, 128, smem);
     if (e != cudaSuccess) return e;
@@ -1352,7 +1353,7 @@ cudaError_t tree_grid(int kind, size_t smem, int* grid)
 template <typename T>
 cudaError_t launch_tree_factor(const DevSched& s, const TreeSched& t, const DevNum<T>& nm, int batch, int* ctr,
                                int* stall, long long spin_limit, int grid, size_t smem, int fused, int u0, int nu,
-                               int tick, cudaStream_t st)
+                               int tick, bool narrow, cudaStream_t st)
 {
     const int g = std::min<long long>(grid, (long long)nu * batch);
     if (g <= 0) return cudaSuccess;
@@ -1361,8 +1362,9 @@ cudaError_t launch_tree_factor(const DevSched& s, const TreeSched& t, const DevN
     if (fused == kFwdInside && (!t.fwd_in || !nm.vin)) return cudaErrorInvalidValue;
     if (u0 < 0 || nu < 0 || u0 + nu > (fused == kFwdUnits ? t.nunits_fused : t.nunits) || (tick != 0 && tick != 3))
         return cudaErrorInvalidValue;
-    tree_factor_entry<false>((const T*)nullptr)<<<g, 256, smem, st>>>(s, t, nm, batch, ctr, stall, spin_limit, fused, u0, nu, tick,
-                                                       nullptr, nullptr, 0);
+    const auto kernel = narrow ? tree_factor_kernel<T, false, kTreeNtNarrow> : tree_factor_kernel<T, false, kTreeNt>;
+    kernel<<<g, narrow ? kTreeNtNarrow : kTreeNt, smem, st>>>(s, t, nm, batch, ctr, stall, spin_limit, fused, u0, nu,
+                                                              tick, nullptr, nullptr, 0);
     return cudaGetLastError();
 }
 
@@ -1373,7 +1375,7 @@ cudaError_t launch_tree_factor_group(const TreeJob<T>* jobs, const TreeSeg* segs
     const int g = std::min(grid, total);
     if (g <= 0) return cudaSuccess;
     if (!jobs || !segs || nseg <= 0 || !gctr) return cudaErrorInvalidValue;
-    tree_factor_entry<true>((const T*)nullptr)<<<g, 256, smem, st>>>(DevSched{}, TreeSched{}, DevNum<T>{}, 1, gctr, nullptr,
+    tree_factor_kernel<T, true, kTreeNt><<<g, kTreeNt, smem, st>>>(DevSched{}, TreeSched{}, DevNum<T>{}, 1, gctr, nullptr,
                                                       spin_limit, 0, 0, total, 0, jobs, segs, nseg);
     return cudaGetLastError();
 }
@@ -1403,7 +1405,8 @@ cudaError_t launch_tree_bwd(const DevSched& s, const TreeSched& t, const DevNum<
 #define KKT_TREE_INST(T)                                                                                          \
     template cudaError_t tree_grid<T>(int, size_t, int*);                                                          \
     template cudaError_t launch_tree_factor<T>(const DevSched&, const TreeSched&, const DevNum<T>&, int, int*,     \
-                                               int*, long long, int, size_t, int, int, int, int, cudaStream_t);    \
+                                               int*, long long, int, size_t, int, int, int, int, bool,             \
+                                               cudaStream_t);                                                      \
     template cudaError_t launch_tree_fwd<T>(const DevSched&, const TreeSched&, const DevNum<T>&, int, int*,        \
                                             long long, int, size_t, cudaStream_t);                                 \
     template cudaError_t launch_tree_bwd<T>(const DevSched&, const TreeSched&, const DevNum<T>&, int, int*,        \
@@ -1425,10 +1428,12 @@ static cudaError_t allow_smem_tree(K kernel, int optin)
 cudaError_t configure_tree_kernels(int optin)
 {
     cudaError_t e;
-    if ((e = allow_smem_tree(tree_factor_entry<false>((const double*)nullptr), optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_entry<false>((const float*)nullptr), optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_entry<true>((const double*)nullptr), optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_entry<true>((const float*)nullptr), optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<double, false, kTreeNt>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<float, false, kTreeNt>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<double, false, kTreeNtNarrow>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<float, false, kTreeNtNarrow>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<double, true, kTreeNt>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_kernel<float, true, kTreeNt>, optin))) return e;
     if ((e = allow_smem_tree(tree_fwd_kernel<double>, optin))) return e;
     if ((e = allow_smem_tree(tree_fwd_kernel<float>, optin))) return e;
     if ((e = allow_smem_tree(tree_bwd_kernel<double>, optin))) return e;
