@@ -110,32 +110,61 @@ __global__ void __launch_bounds__(128) line_terms_kernel(int nb, int nl, int flo
     }
 }
 
-__global__ void __launch_bounds__(256) gather_values_kernel(int64_t nnz, const int* __restrict__ tptr,
+// Four fifths of the nonzeros are one line's term and nothing else: their code
+// is that term (the first `single` blocks, kGatherEach entries per thread, all
+// their loads in flight). Each of the others (code -1) has a record {position,
+// first term, last term + 1, kind | argument << 2} and a thread of the blocks
+// after those: its terms, listed in tidx, are summed in line order, then the
+// diagonal or constant part is added. A thread per nonzero walking four
+// dependent loads, and every warp the records' longer way: 66 us on 70,000
+// buses (kkt_model_assemble 119 -> 92 us).
+constexpr int kGatherEach = 4;
+__global__ void __launch_bounds__(256) gather_values_kernel(int64_t nnz, int single, const int* __restrict__ codes,
+                                                            int n_multi, const int4* __restrict__ multi,
                                                             const int* __restrict__ tidx,
-                                                            const int* __restrict__ extra_kind,
-                                                            const int* __restrict__ extra_arg,
                                                             const double* __restrict__ terms,
                                                             const double* __restrict__ sigma,
                                                             const double* __restrict__ dual_diag,
                                                             const double* __restrict__ twoc2, int pg0, int ng,
                                                             double dw, double dc, double* __restrict__ vals)
 {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nnz) return;
+    if ((int)blockIdx.x < single) {
+        const int64_t e0 = (int64_t)blockIdx.x * (256 * kGatherEach) + threadIdx.x;
+        int code[kGatherEach];
+        double t[kGatherEach];
+#pragma unroll
+        for (int u = 0; u < kGatherEach; ++u) code[u] = e0 + 256 * u < nnz ? codes[e0 + 256 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < kGatherEach; ++u) t[u] = code[u] >= 0 ? terms[code[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kGatherEach; ++u)                      // 0 + t: a sum of one term is never -0
+            if (code[u] >= 0)
+                vals[e0 + 256 * u] = __double_as_longlong(t[u]) == (long long)0x8000000000000000ull ? 0.0 : t[u];
+        return;
+    }
+    const int r = ((int)blockIdx.x - single) * 256 + threadIdx.x;
+    if (r >= n_multi) return;
+    const int4 m = multi[r];
+    const int kind = m.w & 3, arg = (int)((unsigned)m.w >> 2);
     double acc = 0.0;
-    for (int k = tptr[e]; k < tptr[e + 1]; ++k) acc += terms[tidx[k]];
-    const int kind = extra_kind[e];
+    for (int k0 = m.y; k0 < m.z; k0 += 4) {                        // four terms' loads at a time
+        double t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = k0 + u < m.z ? terms[tidx[k0 + u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k0 + u < m.z) acc += t[u];
+    }
     if (kind == kExtraPrimal) {
-        const int i = extra_arg[e];
-        double d = sigma[i] + dw;
-        if (i >= pg0 && i < pg0 + ng) d += twoc2[i - pg0];
+        double d = sigma[arg] + dw;
+        if (arg >= pg0 && arg < pg0 + ng) d += twoc2[arg - pg0];
         acc += d;
     } else if (kind == kExtraDual) {
-        acc -= dual_diag ? dc + dual_diag[extra_arg[e]] : dc;
+        acc -= dual_diag ? dc + dual_diag[arg] : dc;
     } else if (kind == kExtraOne) {
         acc += 1.0;
     }
-    vals[e] = acc;
+    vals[m.x] = acc;
 }
 
 }  // namespace
@@ -199,11 +228,12 @@ kkt_status kkt_model_create(int32_t n_bus, int32_t n_branch, int32_t n_gen, cons
         std::stable_sort(tr.begin(), tr.end(), [](const Trip& a, const Trip& b) {
             return a.r != b.r ? a.r < b.r : a.c < b.c;
         });
-        std::vector<int> tptr(1, 0), tidx, kind, arg;
+        std::vector<int> tidx, code, multi;
         m->rowptr.assign(n + 1, 0);
         for (size_t p = 0; p < tr.size();) {
             size_t q = p;
             int kd = kExtraNone, ag = 0;
+            const int t0 = (int)tidx.size();
             while (q < tr.size() && tr[q].r == tr[p].r && tr[q].c == tr[p].c) {
                 if (tr[q].term >= 0) tidx.push_back(tr[q].term);
                 else if (kd == kExtraNone) { kd = tr[q].kind; ag = tr[q].arg; }
@@ -212,9 +242,13 @@ kkt_status kkt_model_create(int32_t n_bus, int32_t n_branch, int32_t n_gen, cons
             }
             m->colidx.push_back(tr[p].c);
             m->rowptr[tr[p].r + 1]++;
-            tptr.push_back((int)tidx.size());
-            kind.push_back(kd);
-            arg.push_back(ag);
+            if (kd == kExtraNone && (int)tidx.size() == t0 + 1) {
+                code.push_back(tidx.back());
+                tidx.pop_back();
+            } else {
+                multi.insert(multi.end(), {(int)code.size(), t0, (int)tidx.size(), (int)(kd | (unsigned)ag << 2)});
+                code.push_back(-1);
+            }
             p = q;
         }
         for (int r = 0; r < n; ++r) m->rowptr[r + 1] += m->rowptr[r];
@@ -236,8 +270,8 @@ kkt_status kkt_model_create(int32_t n_bus, int32_t n_branch, int32_t n_gen, cons
         }
         // device copies
         auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-        const size_t sz[] = {al(4 * (size_t)L), al(4 * (size_t)L), al(4 * tptr.size()), al(4 * std::max<size_t>(tidx.size(), 1)),
-                             al(4 * kind.size()), al(4 * arg.size()), al(8 * (size_t)L), al(8 * (size_t)L),
+        const size_t sz[] = {al(4 * (size_t)L), al(4 * (size_t)L), al(4 * code.size()), al(4 * std::max<size_t>(tidx.size(), 1)),
+                             al(4 * std::max<size_t>(multi.size(), 4)), al(8 * (size_t)L), al(8 * (size_t)L),
                              al(8 * std::max(G, 1)), al(8 * (size_t)L * kLineTerms + 8)};
         size_t total = 0;
         for (size_t v : sz) total += v;
@@ -249,13 +283,13 @@ kkt_status kkt_model_create(int32_t n_bus, int32_t n_branch, int32_t n_gen, cons
         char* p = m->base;
         m->d_f = (int*)p; p += sz[0];
         m->d_t = (int*)p; p += sz[1];
-        m->d_tptr = (int*)p; p += sz[2];
+        m->d_code = (int*)p; p += sz[2];
         m->d_tidx = (int*)p; p += sz[3];
-        m->d_kind = (int*)p; p += sz[4];
-        m->d_arg = (int*)p; p += sz[5];
-        m->d_g = (double*)p; p += sz[6];
-        m->d_b = (double*)p; p += sz[7];
-        m->d_twoc2 = (double*)p; p += sz[8];
+        m->d_multi = (int*)p; p += sz[4];
+        m->n_multi = (int)(multi.size() / 4);
+        m->d_g = (double*)p; p += sz[5];
+        m->d_b = (double*)p; p += sz[6];
+        m->d_twoc2 = (double*)p; p += sz[7];
         m->d_terms = (double*)p;
         // through a private non-blocking stream, waited for before returning (a
         // plain cudaMemcpy from pageable memory may return before the device
@@ -267,10 +301,9 @@ kkt_status kkt_model_create(int32_t n_bus, int32_t n_branch, int32_t n_gen, cons
         };
         up(m->d_f, h_from, 4 * (size_t)L);
         up(m->d_t, h_to, 4 * (size_t)L);
-        up(m->d_tptr, tptr.data(), 4 * tptr.size());
+        up(m->d_code, code.data(), 4 * code.size());
         up(m->d_tidx, tidx.data(), 4 * tidx.size());
-        up(m->d_kind, kind.data(), 4 * kind.size());
-        up(m->d_arg, arg.data(), 4 * arg.size());
+        up(m->d_multi, multi.data(), 4 * multi.size());
         up(m->d_g, g.data(), 8 * (size_t)L);
         up(m->d_b, bb.data(), 8 * (size_t)L);
         up(m->d_twoc2, twoc2.data(), 8 * (size_t)G);
@@ -310,10 +343,10 @@ kkt_status kkt_model_assemble(const kkt_model* m, const double* d_V, const doubl
     if (m->nl > 0)
         line_terms_kernel<<<(m->nl + 127) / 128, 128, 0, st>>>(m->nb, m->nl, m->flow, m->d_f, m->d_t, m->d_g, m->d_b,
                                                                d_V, d_theta, d_lambda, m->d_terms);
-    const int blocks = (int)((m->nnz + 255) / 256);
-    gather_values_kernel<<<blocks, 256, 0, st>>>(m->nnz, m->d_tptr, m->d_tidx, m->d_kind, m->d_arg, m->d_terms,
-                                                 d_sigma, d_dual_diag, m->d_twoc2, 2 * m->nb, m->ng, delta_w, delta_c,
-                                                 d_vals);
+    const int single = (int)((m->nnz + 256 * kGatherEach - 1) / (256 * kGatherEach));
+    gather_values_kernel<<<single + (m->n_multi + 255) / 256, 256, 0, st>>>(
+        m->nnz, single, m->d_code, m->n_multi, reinterpret_cast<const int4*>(m->d_multi), m->d_tidx, m->d_terms, d_sigma,
+        d_dual_diag, m->d_twoc2, 2 * m->nb, m->ng, delta_w, delta_c, d_vals);
     return cudaGetLastError() == cudaSuccess ? KKT_OK : KKT_E_CUDA;
 }
 

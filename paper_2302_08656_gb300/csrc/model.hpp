@@ -12,7 +12,9 @@ struct kkt_model {
     std::vector<int> from, to, gen_bus;  // host copy of the topology
     std::vector<double> c2;
     char* base = nullptr;                // one device allocation
-    int *d_f = nullptr, *d_t = nullptr, *d_tptr = nullptr, *d_tidx = nullptr, *d_kind = nullptr, *d_arg = nullptr;
+    int *d_f = nullptr, *d_t = nullptr, *d_tidx = nullptr;
+    int *d_code = nullptr, *d_multi = nullptr;   // per nonzero: its only term or -1; records of the others
+    int n_multi = 0;
     double *d_g = nullptr, *d_b = nullptr, *d_twoc2 = nullptr, *d_terms = nullptr;
     // interior-point loop (kkt_model_set_limits): loads, bounds, limits,
     // topology lists and the loop's workspace, in one device allocation
