@@ -191,7 +191,7 @@ template <bool FULL, int NW>
 __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, int pk, float floorT, int& n_bad,
                                               int& n_pert)
 {
-    constexpr int kPanel = 8;
+    constexpr int kPanel = 8, NC = NW == 8 ? 3 : 32 / NW;      // columns of a warp in flight
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int row = p0 + tx;
     if (ty == 0) {
@@ -210,22 +210,22 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
     float lp[kPanel];
 #pragma unroll
     for (int k = 0; k < kPanel; ++k) lp[k] = ((FULL || k < pk) && row < Fr) ? M[row + (p0 + k) * Fr] : 0.0f;
-    for (int jb = p0 + pk + ty; jb < Fc; jb += 3 * NW) {
-        float v[3];
+    for (int jb = p0 + pk + ty; jb < Fc; jb += NC * NW) {
+        float v[NC];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] = (row < Fr && jb + NW * c < Fc) ? M[row + (jb + NW * c) * Fr] : 0.0f;
+        for (int c = 0; c < NC; ++c) v[c] = (row < Fr && jb + NW * c < Fc) ? M[row + (jb + NW * c) * Fr] : 0.0f;
 #pragma unroll
         for (int k = 0; k < kPanel; ++k) {
             if (!FULL && k >= pk) break;                           // warp-uniform
             const bool upd = tx > k;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
+            for (int c = 0; c < NC; ++c) {
                 const float u = __shfl_sync(0xffffffffu, v[c], k);   // row p0 + k: final at step k
                 if (upd) v[c] -= lp[k] * u;
             }
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < NC; ++c)
             if (row < Fr && jb + NW * c < Fc) M[row + (jb + NW * c) * Fr] = v[c];
     }
     __syncthreads();
@@ -547,7 +547,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             }
             __syncthreads();
             // group of warp ty: the last ones to the warps that share warp 0's sub-partition
-            constexpr int CG = NW == 8 ? 5 : 2;
+            constexpr int CG = NW == 8 ? 5 : 32 / NW;
             const int g = ty & 3 ? ty / 4 * 3 + (ty & 3) - 1 : NW / 4 * 3 + ty / 4 - 1;
             for (int p = 0; p < w; ++p) {
                 const int i = p + 1 + tx;
