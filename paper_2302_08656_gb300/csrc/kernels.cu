@@ -454,8 +454,8 @@ __device__ __forceinline__ double sell_row_dot(const DevSched& s, const SellSeg&
 // static pivot and its reciprocal (pivot_rcp's value: the Newton step, the
 // division outside its range). The static-pivot events are accumulated in
 // bad / pert and counted once per front by the caller. Single precision
-// only: measured on GB300, FP64 instructions cost pipe time per active lane,
-// so in double precision one lane computes the pivot and shares it.
+// only: in double precision one lane computes the pivot and shares it (the
+// select of the static pivot alone is 150 cycles there, on every lane's path).
 template <typename T>
 __device__ __forceinline__ T uniform_pivot(T x, T floorT, T& r, bool& bad, int& pert)
 {
@@ -498,8 +498,9 @@ __device__ __forceinline__ void assemble_original(const DevSched& s, const DevNu
 
 // The loops of the leaf and warp front kernels are kept rolled: they run once or
 // a few times each, and unrolled fourfold the kernels were 24 to 43 KB of code
-// (now 10 to 27): 64 scenarios of 2,000 buses FP32 1310 -> 1237 us, 70,000
-// buses FP32 1612 -> 1605, FP64 2700 -> 2693.
+// (now 10 to 27): 70,000 buses FP32 1612 -> 1605 us, FP64 2700 -> 2693; 64
+// scenarios of 2,000 buses FP32, together with the copied factors of the
+// substitutions below, 1314 -> 1237.
 //
 // Loops over the entries of dense blocks use fixed two-dimensional thread
 // layouts (rows across lanes, columns across lane groups or warps), so no
@@ -1144,12 +1145,11 @@ __global__ void solve_post_kernel(int n, const int* __restrict__ perm, DevNum<T>
 // dimension w <= G, in shared memory) by a group of G lanes (gmask, lane gl
 // of the group holding v_gl in a register, the pivot entry broadcast by a
 // shuffle); the operations and their order are those of the shared-memory
-// loop x_p = v_p * (1 / u_pp), v_a -= u_ap x_p (the bits are the same). FP64
-// costs pipe time per active lane, so the reciprocals are formed by all lanes
-// at once before the dependent chain, and on the chain each step is one
-// lane's multiply and the FMAs of the lanes above the pivot (instead of a
-// reciprocal and a multiply on every lane per step: 0.184 -> 0.165 ms of
-// solve_bwd_kernel per 70k FP64 solve). A register version of the forward
+// loop x_p = v_p * (1 / u_pp), v_a -= u_ap x_p (the bits are the same). The
+// reciprocals are formed by all lanes at once before the dependent chain, and
+// on the chain each step is a multiply and an FMA (instead of a reciprocal and
+// a multiply per step: 0.184 -> 0.165 ms of solve_bwd_kernel per 70k FP64
+// solve). A register version of the forward
 // block was slower on the wide levels (more instructions per front) and is
 // not used there.
 template <typename T, int G>

@@ -510,23 +510,24 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                 if (tx == 0 && n_pert) atomicAdd(&nm.stat->n_perturbed, n_pert);
             }
         } else if (sizeof(T) == 8 && Fr <= 32 && Fc <= 32) {
-            // mini fronts of at most 32 x 32 (always when w <= 16). GB300 runs
-            // one FP64 warp instruction per ~64 cycles per sub-partition, masked
-            // lanes included, so the elimination is bound by the FP64
-            // instructions issued. Warp 0 owns column p+1 only: at step p it
-            // finishes the next pivot (lane 0), broadcasts its reciprocal and
-            // stores column p+1 already scaled, so at step p+1 every other warp
-            // reads l_i,p+1 and issues FMAs alone. The other warps own CG adjacent
-            // columns each from p+2 (lane -> row), a warp whose columns are all
-            // eliminated issues nothing, and warp 4, which shares a
-            // sub-partition with warp 0, takes the last group.
+            // mini fronts of at most 32 x 32 (always when w <= 16). On GB300 a
+            // warp starts one FP64 instruction per 64 cycles and the SM one per
+            // 19, masked lanes included, so the elimination is bound by the
+            // FP64 instructions issued. Warp 0 owns column p+1 only: at step p
+            // it finishes the next pivot and stores column p+1 already scaled,
+            // so at step p+1 every other warp reads l_i,p+1 and issues FMAs
+            // alone. The other warps own CG adjacent columns each from p+2
+            // (lane -> row), a warp whose columns are all eliminated issues
+            // nothing, and the warps that share warp 0's sub-partition take
+            // the last groups.
             // A pivot is computed by every lane of warp 0 from lane 0's entry
             // (one lane alone: 46 cycles of divergence), and its reciprocal
             // starts at once: that the entry is kept as it is and in the
             // range of the Newton step is tested on its high word beside it
-            // (lo, hi), and pivot_slow repeats the rare others. A pivot's
-            // chain, update, reciprocal, scaling and exchanges, is 430 cycles
-            // so, 630 with the static pivot and the range test in it.
+            // (lo, hi), and pivot_slow repeats the rare others. A dependent
+            // pivot step took 630 cycles with the static pivot and the range
+            // test in it, 476 with the tests apart (one warp); refactor_refine
+            // 25,000 buses FP64 1367 -> 1326 us, 9,973 999 -> 965.
             unsigned lo = (unsigned)__double2hiint((double)floorT) + 1u;   // above it: not below the floor
             lo = lo > (23u << 20) ? lo : 23u << 20;                // pivot_rcp_fast_ok: biased exponents 23 .. 2023
             const unsigned hi = (2023u << 20) | 0xfffffu;
@@ -681,9 +682,12 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
     }
 }
 
-// Entry points, NT threads per CTA. kTreeNt on the wide levels: in single
-// precision held to 64 registers, so that 4 CTAs fit on an SM, in double
-// precision to 80, for 3. The narrow top of the tree, one CTA per SM, takes
+// Entry points, NT threads per CTA. kTreeNt on the wide levels, held to 64
+// registers, so that 4 CTAs fit on an SM (in double precision 80 registers and
+// 3 CTAs: 25,000 buses 1282 -> 1299 us per refactor_refine, 70,000 2622 -> 2639;
+// in single precision 5 CTAs were slower). The narrow top of the tree, one CTA
+// per SM (a level is narrow with at most one unit per SM; with two: 25,000 buses
+// FP32 877 -> 896 us, 70,000 1599 -> 1643), takes
 // kTreeNtNarrow threads: a warp starts one FP64 instruction per 64 cycles, so
 // with 7 warps and 5 columns each the trailing update of a pivot took 726
 // cycles against 520 of the pivot's own chain; 15 warps take 2 columns each, and
@@ -693,7 +697,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
 // buses FP32 1759 -> 1863, FP64 2957 -> 3149.)
 constexpr int kTreeNt = 256, kTreeNtNarrow = 512;
 template <typename T, bool MULTI, int NT>
-__global__ void __launch_bounds__(NT, NT == kTreeNtNarrow ? 1 : sizeof(T) == 4 ? 4 : 3)
+__global__ void __launch_bounds__(NT, NT == kTreeNtNarrow ? 1 : 4)
 tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr, int* stall, long long limit, int fused,
                    int u0, int nu, int tick, const TreeJob<T>* jobs, const TreeSeg* segs, int nseg)
 {
