@@ -1846,8 +1846,10 @@ kkt_status kkt_residual(kkt_ctx* c, const double* d_rhs, const double* d_x, doub
     // the residual and the four maxima in one pass and one read: three norms of
     // two launches and a synchronization each, and a read of ||K||, took most
     // of the call (25,000 buses 118 -> 39 us)
-    KKT_CUDA(launch_resid_omega(c->sched, c->last_vals, c->slots, d_x, d_rhs, d_r, c->omega_part, c->stat,
-                                c->omega_dev, 1, st, c->red));
+    // scratch: the refinement's (partial maxima in V, results in red), as the
+    // norms before, so that a checked solve under way keeps its own
+    KKT_CUDA(launch_resid_omega(c->sched, c->last_vals, c->slots, d_x, d_rhs, d_r, c->V, c->stat, c->red + 8, 1, st,
+                                c->red));
     KKT_CUDA(cudaMemcpyAsync(c->pin, c->red, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
     KKT_CUDA(cudaStreamSynchronize(st));
     const double rm = c->pin[0], xm = c->pin[1], bm = c->pin[2], knorm = c->pin[3];
