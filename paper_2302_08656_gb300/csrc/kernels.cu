@@ -729,9 +729,9 @@ __global__ void __launch_bounds__(128, 8) front_warp_kernel(DevSched s, DevNum<T
             if (lane > p && lane < F) Fm[lane + p * F] *= r;
         } else {
             if (lane == 0) {
-                const T pv = static_pivot(Fm[p + p * F], floorT, nm.stat, true);
-                Fm[p + p * F] = pv;
-                srinv[wid] = pivot_rcp(pv);
+                double r;
+                Fm[p + p * F] = fast_pivot(Fm[p + p * F], floorT, nm.stat, true, r);
+                srinv[wid] = r;
             }
             __syncwarp();
             if (lane > p && lane < F) Fm[lane + p * F] *= srinv[wid];
@@ -811,9 +811,9 @@ __global__ void __launch_bounds__(128) front_leaf_kernel(DevSched s, DevNum<T> n
             if (gl > p && gl < F) Fm[gl + p * F] *= r;
         } else {
             if (gl == 0) {
-                const T pv = static_pivot(Fm[p + p * F], floorT, nm.stat, true);
-                Fm[p + p * F] = pv;
-                srinv[slot] = pivot_rcp(pv);
+                double r;
+                Fm[p + p * F] = fast_pivot(Fm[p + p * F], floorT, nm.stat, true, r);
+                srinv[slot] = r;
             }
             __syncwarp(gmask);
             if (gl > p && gl < F) Fm[gl + p * F] *= srinv[slot];
@@ -895,9 +895,9 @@ __global__ void __launch_bounds__(256) front_cta_kernel(DevSched s, DevNum<T> nm
             if (tid == 0) Fm[p + p * F] = pv;
         } else {
             if (tid == 0) {
-                const T pv = static_pivot(Fm[p + p * F], floorT, nm.stat, true);
-                Fm[p + p * F] = pv;
-                srinv = pivot_rcp(pv);
+                double r;
+                Fm[p + p * F] = fast_pivot(Fm[p + p * F], floorT, nm.stat, true, r);
+                srinv = r;
             }
             __syncthreads();
             const T rinv = srinv;
@@ -1014,9 +1014,9 @@ __global__ void __launch_bounds__(256) front_panel_kernel(DevSched s, DevNum<T> 
             if (tid == 0) col[p + (int64_t)p * F] = pv;
         } else {
             if (tid == 0) {
-                const T pv = static_pivot(col[p + (int64_t)p * F], floorT, nm.stat, true);
-                col[p + (int64_t)p * F] = pv;
-                srinv = pivot_rcp(pv);
+                double r;
+                col[p + (int64_t)p * F] = fast_pivot(col[p + (int64_t)p * F], floorT, nm.stat, true, r);
+                srinv = r;
             }
             __syncthreads();
             const T rinv = srinv;

@@ -231,15 +231,6 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
     __syncthreads();
 }
 
-// A pivot of the double-precision elimination that is not simply kept with its
-// Newton reciprocal (r, unused: see pivot_rcp_div): static pivoting, then
-// pivot_rcp. Returns the pivot and its reciprocal; counts the event if count.
-__device__ __noinline__ double2 pivot_slow(double x, double, double floorT, DevStat* stat, bool count)
-{
-    const double pv = static_pivot(x, floorT, stat, count);
-    return make_double2(pv, pivot_rcp(pv));
-}
-
 // ------------------------------------------------------------- refactor
 
 // Unit (q, ti, tj) of instance b. Mini front M (Fr x Fc, column-major, ld Fr):
@@ -523,22 +514,11 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             // A pivot is computed by every lane of warp 0 from lane 0's entry
             // (one lane alone: 46 cycles of divergence), and its reciprocal
             // starts at once: that the entry is kept as it is and in the
-            // range of the Newton step is tested on its high word beside it
-            // (lo, hi), and pivot_slow repeats the rare others. A dependent
+            // range of the Newton step is tested beside it (fast_pivot). A dependent
             // pivot step took 630 cycles with the static pivot and the range
             // test in it, 476 with the tests apart (one warp); refactor_refine
             // 25,000 buses FP64 1367 -> 1326 us, 9,973 999 -> 965.
-            unsigned lo = (unsigned)__double2hiint((double)floorT) + 1u;   // above it: not below the floor
-            lo = lo > (23u << 20) ? lo : 23u << 20;                // pivot_rcp_fast_ok: biased exponents 23 .. 2023
-            const unsigned hi = (2023u << 20) | 0xfffffu;
-            auto pivot = [&](double x, double& r) {
-                r = pivot_rcp_fast(x);
-                const unsigned ax = (unsigned)__double2hiint(x) & 0x7fffffffu;
-                if (ax >= lo && ax <= hi) return x;                // warp-uniform
-                const double2 q = pivot_slow(x, r, (double)floorT, nm.stat, lead && tx == 0);
-                r = q.y;
-                return q.x;
-            };
+            auto pivot = [&](double x, double& r) { return fast_pivot(x, (double)floorT, nm.stat, lead && tx == 0, r); };
             if (ty == 0 && w > 0) {
                 double r;
                 const T pv = (T)pivot((double)M[0], r);
