@@ -377,6 +377,14 @@ cudaError_t launch_solve_post(const DevSched& s, const DevNum<T>& nm, double* x,
 // K the sliced copy (instance stride bs_slot); part holds batch * resid_blocks(n) * 4 doubles
 constexpr int kResidRows = 32;         // a block has at least one slice of 32 rows (bounds the partial-maxima buffer)
 inline int resid_blocks(int n) { return (n + kResidRows - 1) / kResidRows; }
+// The doubles of the Krylov basis V of one instance: restart + 1 vectors, and
+// room for the partial maxima that kkt_residual keeps there (more than the
+// vectors for n = 1, restart = 1).
+inline int64_t krylov_doubles(int n, int restart)
+{
+    const int64_t basis = (int64_t)n * (restart + 1), part = 4 * (int64_t)resid_blocks(n);
+    return basis > part ? basis : part;
+}
 // ||K||_inf of every instance is read from stat[inst].knorm_bits (the refactorization's scaling pass);
 // maxima (optional): ||r||, ||x||, ||b||, ||K|| of each instance
 cudaError_t launch_resid_omega(const DevSched& s, const double* kvals, int64_t bs_slot, const double* x,

@@ -1220,7 +1220,7 @@ static int64_t plan_bytes(const Analysis& an, int n, int64_t nnz, const kkt_opti
     add(B * n * es); add(B * std::max<int64_t>((int64_t)an.rel.size(), 1) * es);
     if (tp.ts.fwd_in) add(B * n * es);
     add(B * scratch * es);
-    add((int64_t)n * (o.restart + 1) * 8); add((int64_t)n * o.restart * 8); add(n * 8); add(n * 8);
+    add(krylov_doubles(n, o.restart) * 8); add((int64_t)n * o.restart * 8); add(n * 8); add(n * 8);
     add((int64_t)(kRedScratch + 4096 + 8) * 8);
     add((int64_t)(8 + 2 * (kMaxRestart + 2)) * 8);
     add((int64_t)kGmSize * 8);
@@ -1421,7 +1421,7 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     char* cbv = P.take<char>(B * cbv_unit * es);
     char* vin = tp.ts.fwd_in ? P.take<char>(B * n * es) : nullptr;
     c->panel_scratch = P.take<char>(B * scratch * es);
-    c->V = P.take<double>((int64_t)n * (c->opt.restart + 1));
+    c->V = P.take<double>(krylov_doubles(n, c->opt.restart));
     c->Z = P.take<double>((int64_t)n * c->opt.restart);
     c->w = P.take<double>(n);
     c->r = P.take<double>(n);
