@@ -1848,8 +1848,11 @@ kkt_status kkt_residual(kkt_ctx* c, const double* d_rhs, const double* d_x, doub
     // of the call (25,000 buses 118 -> 39 us)
     // scratch: the refinement's (partial maxima in V, results in red), as the
     // norms before, so that a checked solve under way keeps its own
-    KKT_CUDA(launch_resid_omega(c->sched, c->last_vals, c->slots, d_x, d_rhs, d_r, c->V, c->stat, c->red + 8, 1, st,
-                                c->red));
+    {
+        Launch L(c, st, KK_SPMV, 2);
+        KKT_CUDA(launch_resid_omega(c->sched, c->last_vals, c->slots, d_x, d_rhs, d_r, c->V, c->stat, c->red + 8, 1,
+                                    st, c->red));
+    }
     KKT_CUDA(cudaMemcpyAsync(c->pin, c->red, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
     KKT_CUDA(cudaStreamSynchronize(st));
     const double rm = c->pin[0], xm = c->pin[1], bm = c->pin[2], knorm = c->pin[3];
