@@ -121,9 +121,9 @@ __device__ __forceinline__ double pivot_rcp_fast(double d)
     const double e = fma(-d, x0, 1.0);
     return fma(x0, fma(e, e, e), x0);
 }
-// The division itself is a function of its own: inlined, the compiler puts its
-// six FP64 instructions in front of the range test (114 of the 630 cycles of a
-// pivot). It takes the fast value, which so is formed before the test.
+// The division itself is a function of its own, called for a pivot outside the
+// range only, so that a pivot in the range does not wait for it. It takes the
+// fast value, which so is formed before the test.
 static __device__ __noinline__ double pivot_rcp_div(double d, double) { return 1.0 / d; }
 __device__ __forceinline__ double pivot_rcp(double d)
 {
@@ -186,8 +186,9 @@ __device__ __forceinline__ float static_pivot(float piv, float floorT, DevStat* 
 // A pivot with its reciprocal in double precision: the Newton step starts at
 // once, and whether the entry is kept (not below the floor) and in that step's
 // range is tested beside it, on the high word. pivot_slow takes the rare others
-// (r, unused: see pivot_rcp_div); the event is counted if count. In a chain of
-// pivots the tests in front of the reciprocal were 222 of 630 cycles.
+// (r, unused: see pivot_rcp_div); the event is counted if count. A step of a
+// chain of pivots by one warp took 476 cycles so, 630 with the tests in front
+// of the reciprocal and the division inlined (clock64).
 static __device__ __noinline__ double2 pivot_slow(double x, double, double floorT, DevStat* stat, bool count)
 {
     const double pv = static_pivot(x, floorT, stat, count);
