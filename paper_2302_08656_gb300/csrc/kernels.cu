@@ -2052,6 +2052,18 @@ cudaError_t configure_kernels()
     if ((e = allow_smem(solve_bwd_cta_kernel<float>, optin))) return e;
     if ((e = allow_smem(schur_tile_kernel<double>, optin))) return e;
     if ((e = allow_smem(schur_tile_kernel<float>, optin))) return e;
+    // The two leaf classes of a level run side by side in the captured graphs.
+    // An SM splits its 256 KB between L1 and shared memory by the kernel that
+    // starts on it and keeps that split while the kernel runs: in double
+    // precision the groups of 16 rows (17 KB a CTA) then met the split of the
+    // groups of 8 (9 KB), had few CTAs per SM and took 41 us instead of 14
+    // (2,003 buses; a step 497 us, side by side and one split 447). In single
+    // precision the default split serves both, and the largest cost 3 % where
+    // several contexts work at once (less L1).
+    if ((e = cudaFuncSetAttribute(front_leaf_kernel<double, 8>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared))) return e;
+    if ((e = cudaFuncSetAttribute(front_leaf_kernel<double, 16>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared))) return e;
     return configure_tree_kernels(optin);
 }
 
