@@ -265,7 +265,7 @@ struct TreeFront {
 struct TreeUnit {
     TreeFront d;
     FrontTile u;
-    int pad;
+    int keep;                    // CTAs that the units after this one's level can use (narrow launch; >= 1)
 };
 struct TreeKid {
     int q;                       // tree index of the child, -1 if the child lies below the tree part

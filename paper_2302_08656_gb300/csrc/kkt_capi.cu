@@ -1520,9 +1520,11 @@ static kkt_status analyze_impl(int32_t n, int32_t n_primal, const int32_t* h_row
     e = e ? e : up(tkid, tp.kid.data(), tp.kid.size() * sizeof(TreeKid));
     // units with their fronts' descriptors
     std::vector<TreeUnit> h_unit(tp.unit.size()), h_unit_fused(tp.unit_fused.size());
-    for (size_t i = 0; i < tp.unit.size(); ++i) h_unit[i] = TreeUnit{tp.fr[tp.unit[i].front], tp.unit[i], 0};
+    auto keep_of = [&](int keep) { return (int)std::min<int64_t>(keep * B, 1 << 30); };   // over all instances
+    for (size_t i = 0; i < tp.unit.size(); ++i)
+        h_unit[i] = TreeUnit{tp.fr[tp.unit[i].front], tp.unit[i], keep_of(tp.keep[i])};
     for (size_t i = 0; i < tp.unit_fused.size(); ++i)
-        h_unit_fused[i] = TreeUnit{tp.fr[tp.unit_fused[i].front], tp.unit_fused[i], 0};
+        h_unit_fused[i] = TreeUnit{tp.fr[tp.unit_fused[i].front], tp.unit_fused[i], keep_of(tp.keep_fused[i])};
     e = e ? e : up(tunit, h_unit.data(), h_unit.size() * sizeof(TreeUnit));
     e = e ? e : up(tunit_fused, h_unit_fused.data(), h_unit_fused.size() * sizeof(TreeUnit));
     e = e ? e : up(tinv, tp.inv.data(), tp.inv.size() * 4);

@@ -248,12 +248,15 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
 // Tickets and the abort flag come from the group's counter block (ctr);
 // completion counters are each context's own. The descriptors of the current
 // unit's context are cached in shared memory.
-template <typename T, bool MULTI, int NT>
+constexpr int kTreeNt = 256, kTreeNtNarrow = 512;              // threads per CTA (tree_factor_kernel)
+
+template <typename T, bool MULTI, int NT, int PER>
 __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, DevNum<T> nm0_p, int B_p, int* ctr,
                                                  int* stall, long long limit, int fused, int u0, int nu, int tick,
                                                  const TreeJob<T>* jobs, const TreeSeg* segs, int nseg)
 {
     constexpr int NW = NT / 32, KC = 32 / NW;                  // warps; columns of a thread
+    constexpr bool AHEAD = sizeof(T) == 8 && !(NT == kTreeNtNarrow && PER == 2);
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ TreeUnit su;                                    // the current unit and its front
     TreeFront& d = su.d;
@@ -266,7 +269,11 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
     const int total = MULTI ? nu : nu * B_p;
     __shared__ int s_cut[kTreeMaxKids + 1];
     if (MULTI && tid == 0) s_job = -1;
+    int keep = 1 << 30;
     for (;;) {
+        // a CTA beyond what the levels above its last unit can use leaves its
+        // place on the SM to other contexts' work; block 0 stays to the end
+        if (NT == kTreeNtNarrow && (int)blockIdx.x >= keep) break;
         const int t = next_ticket(ctr + tick, ctr + 1, total, &s_t);
         if (t >= total) break;
         int ul, b;
@@ -315,6 +322,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         copy_words(&su, units + (MULTI ? 0 : u0) + ul, 1, tid, NT);
         __syncthreads();
         const FrontTile ut = su.u;
+        keep = su.keep;
         const int q = ut.front;
         const DevNum<T> nm = nm0.at(b);
         if (ut.ti < 0) {                                           // forward-solve unit (fused mode)
@@ -364,10 +372,13 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
         T xf = T(0);
         if (fwd_here && tid < w) xf = nm.vin[d.first + tid];       // w <= 32; vin: the lead unit overwrites vec
         // where a thread's first children's entries are (kAhead per column):
-        // found before the wait, so that the loads are issued right after it
-        // (with partial pivot panels of their own length, below: 70k buses
-        // FP32 step 1691 -> 1666 us, FP64 2891 -> 2793)
-        const bool ahead = ts.cb32 && Fr <= 32 && Fc <= 32 && nk <= 32;
+        // found before the wait, so that the loads are issued right after it.
+        // Double precision only, and not in the narrow form of two CTAs per SM:
+        // where the registers are held to 64 it costs more than it gives
+        // (refactor_refine FP32 with it and without, 9,973 buses 555 and 532
+        // us, 25,000 828 and 792; FP64, in the wide launch alone, 70,000 buses
+        // 2617 and 2645)
+        const bool ahead = AHEAD && ts.cb32 && Fr <= 32 && Fc <= 32 && nk <= 32;
         constexpr int kAhead = 2;
         constexpr unsigned kNone = 0xffffffffu;
         T acc[KC];
@@ -667,22 +678,40 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
 // 3 CTAs: 25,000 buses 1282 -> 1299 us per refactor_refine, 70,000 2622 -> 2639;
 // in single precision 5 CTAs were slower). The narrow top of the tree, one CTA
 // per SM (a level is narrow with at most one unit per SM; with two: 25,000 buses
-// FP32 877 -> 896 us, 70,000 1599 -> 1643), takes
-// kTreeNtNarrow threads: a warp starts one FP64 instruction per 64 cycles, so
-// with 7 warps and 5 columns each the trailing update of a pivot took 726
-// cycles against 520 of the pivot's own chain; 15 warps take 2 columns each, and
-// loads and gathers have twice the threads. refactor_refine 200 buses FP64 300
-// -> 283 us, 2,003 FP32 347 -> 329, 9,973 FP64 967 -> 943, 25,000 FP64 1331 ->
-// 1304, FP32 920 -> 883. (The wide levels with 128 threads, twice the CTAs: 70,000
-// buses FP32 1759 -> 1863, FP64 2957 -> 3149.)
-constexpr int kTreeNt = 256, kTreeNtNarrow = 512;
-template <typename T, bool MULTI, int NT>
-__global__ void __launch_bounds__(NT, NT == kTreeNtNarrow ? 1 : 4)
+// FP32 877 -> 896 us, 70,000 1599 -> 1643), takes kTreeNtNarrow threads: a warp
+// starts one FP64 instruction per 64 cycles, so with 7 warps and 5 columns each
+// the trailing update of a pivot took 726 cycles against 520 of the pivot's own
+// chain; 15 warps take 2 columns each, and loads and gathers have twice the
+// threads (refactor_refine with 256 and with 512 threads: 200 buses FP64 300 and
+// 283 us, 9,973 967 and 943, 25,000 1331 and 1304).
+//
+// PER: the CTAs of 512 threads that an SM must hold. With the compiler's choice
+// of 103 registers one of them fills an SM, and contexts that refactor at the
+// same time (kkt_refactor_batched, streams of their own) queue for the SMs: 16
+// contexts of 2,003 buses FP32 862 -> 1253 us, FP64 1414 -> 1679, of 9,973 FP32
+// 3027 -> 4438. Held to 64 registers two fit, beside 256-thread CTAs of other
+// contexts, and a CTA leaves once the levels above cannot use it (TreeUnit::
+// keep; without leaving 935 us and 1297): 776, 1046 and 3080 us. Single
+// precision always takes that form (a lone context: no difference without the
+// gather ahead of the wait). In double precision it costs a lone
+// refactor_refine 1 to 4 % (200 buses 275 -> 282 us, 2,003 450 -> 463, 9,973
+// 766 -> 783), so that call, which waits for its result, keeps the form of one
+// CTA per SM, and kkt_refactor, which does not, takes the form of two.
+template <typename T, bool MULTI, int NT, int PER>
+__global__ void __launch_bounds__(NT, PER)
 tree_factor_kernel(DevSched s, TreeSched ts, DevNum<T> nm, int B, int* ctr, int* stall, long long limit, int fused,
                    int u0, int nu, int tick, const TreeJob<T>* jobs, const TreeSeg* segs, int nseg)
 {
-    tree_factor_body<T, MULTI, NT>(s, ts, nm, B, ctr, stall, limit, fused, u0, nu, tick, jobs, segs, nseg);
+    tree_factor_body<T, MULTI, NT, PER>(s, ts, nm, B, ctr, stall, limit, fused, u0, nu, tick, jobs, segs, nseg);
 }
+template <typename T>
+constexpr auto tree_factor_wide = tree_factor_kernel<T, false, kTreeNt, 4>;
+template <typename T>
+constexpr auto tree_factor_multi = tree_factor_kernel<T, true, kTreeNt, 4>;
+template <typename T>
+constexpr auto tree_factor_narrow = tree_factor_kernel<T, false, kTreeNtNarrow, 2>;      // shares the SMs
+template <typename T>
+constexpr auto tree_factor_alone = tree_factor_kernel<T, false, kTreeNtNarrow, sizeof(T) == 8 ? 1 : 2>;
 
 // ------------------------------------------------------ forward substitution
 
@@ -1316,8 +1345,8 @@ cudaError_t tree_grid(int kind, size_t smem, int* grid)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
-    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_kernel<T, false, kTreeNt>, kTreeNt, smem);
-    else if (kind == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_kernel<T, true, kTreeNt>, kTreeNt, smem);
+    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_wide<T>, kTreeNt, smem);
+    else if (kind == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_multi<T>, kTreeNt, smem);
     else if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_fwd_kernel<T>, 128, smem);
     else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_bwd_kernel<T>, 128, smem);
     if (e != cudaSuccess) return e;
@@ -1346,7 +1375,7 @@ cudaError_t launch_tree_factor(const DevSched& s, const TreeSched& t, const DevN
     if (fused == kFwdInside && (!t.fwd_in || !nm.vin)) return cudaErrorInvalidValue;
     if (u0 < 0 || nu < 0 || u0 + nu > (fused == kFwdUnits ? t.nunits_fused : t.nunits) || (tick != 0 && tick != 3))
         return cudaErrorInvalidValue;
-    const auto kernel = narrow ? tree_factor_kernel<T, false, kTreeNtNarrow> : tree_factor_kernel<T, false, kTreeNt>;
+    const auto kernel = !narrow ? tree_factor_wide<T> : fused != kFwdNone ? tree_factor_alone<T> : tree_factor_narrow<T>;
     kernel<<<g, narrow ? kTreeNtNarrow : kTreeNt, smem, st>>>(s, t, nm, batch, ctr, stall, spin_limit, fused, u0, nu,
                                                               tick, nullptr, nullptr, 0);
     return cudaGetLastError();
@@ -1359,8 +1388,8 @@ cudaError_t launch_tree_factor_group(const TreeJob<T>* jobs, const TreeSeg* segs
     const int g = std::min(grid, total);
     if (g <= 0) return cudaSuccess;
     if (!jobs || !segs || nseg <= 0 || !gctr) return cudaErrorInvalidValue;
-    tree_factor_kernel<T, true, kTreeNt><<<g, kTreeNt, smem, st>>>(DevSched{}, TreeSched{}, DevNum<T>{}, 1, gctr, nullptr,
-                                                      spin_limit, 0, 0, total, 0, jobs, segs, nseg);
+    tree_factor_multi<T><<<g, kTreeNt, smem, st>>>(DevSched{}, TreeSched{}, DevNum<T>{}, 1, gctr, nullptr, spin_limit, 0,
+                                                   0, total, 0, jobs, segs, nseg);
     return cudaGetLastError();
 }
 
@@ -1412,12 +1441,13 @@ static cudaError_t allow_smem_tree(K kernel, int optin)
 cudaError_t configure_tree_kernels(int optin)
 {
     cudaError_t e;
-    if ((e = allow_smem_tree(tree_factor_kernel<double, false, kTreeNt>, optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_kernel<float, false, kTreeNt>, optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_kernel<double, false, kTreeNtNarrow>, optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_kernel<float, false, kTreeNtNarrow>, optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_kernel<double, true, kTreeNt>, optin))) return e;
-    if ((e = allow_smem_tree(tree_factor_kernel<float, true, kTreeNt>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_wide<double>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_wide<float>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_narrow<double>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_alone<double>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_narrow<float>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_multi<double>, optin))) return e;
+    if ((e = allow_smem_tree(tree_factor_multi<float>, optin))) return e;
     if ((e = allow_smem_tree(tree_fwd_kernel<double>, optin))) return e;
     if ((e = allow_smem_tree(tree_fwd_kernel<float>, optin))) return e;
     if ((e = allow_smem_tree(tree_bwd_kernel<double>, optin))) return e;

@@ -7,6 +7,17 @@ namespace kktgb {
 
 static size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
+// TreePlan::keep of an order that ascends by level (lev: level of each tree index).
+static void keep_counts(const std::vector<FrontTile>& order, const std::vector<int>& lev, int n_levels,
+                        std::vector<int>& keep)
+{
+    std::vector<int> cnt(n_levels + 1, 0), above(n_levels + 2, 1);
+    for (const FrontTile& u : order) cnt[lev[u.front]]++;
+    for (int l = n_levels - 1; l >= 0; --l) above[l] = std::max(above[l + 1], cnt[l] + cnt[l + 1]);
+    keep.clear();
+    for (const FrontTile& u : order) keep.push_back(above[lev[u.front] + 1]);
+}
+
 void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
 {
     tp = TreePlan();
@@ -138,6 +149,13 @@ void build_tree(const Analysis& an, int min_fronts, size_t es, TreePlan& tp)
         for (int q = q0; q < q1; ++q) tp.unit_fused.push_back(FrontTile{q, -1, 0});
     }
     ts.nunits_fused = (int)tp.unit_fused.size();
+    {
+        std::vector<int> lev(nq);
+        for (int l = split; l < an.n_levels; ++l)
+            for (int s : order[l]) lev[tq[s]] = l;
+        keep_counts(tp.unit, lev, an.n_levels, tp.keep);
+        keep_counts(tp.unit_fused, lev, an.n_levels, tp.keep_fused);
+    }
     ts.max_kids = std::max(ts.max_kids, 1);
     ts.kid_pitch = ts.max_kids | 1;
     ts.fwd_in = ts.map_w <= 32 ? 1 : 0;

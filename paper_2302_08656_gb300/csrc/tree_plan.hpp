@@ -22,6 +22,10 @@ struct TreePlan {
     std::vector<TreeKid> kid;
     std::vector<FrontTile> unit;
     std::vector<FrontTile> unit_fused;  // factor units and, after each level, its forward-solve units (ti = -1)
+    // per unit of either order: the most units that any two adjacent levels
+    // above the unit's own have together, at least 1: as many CTAs keep every
+    // unit of a level at work while those of the next are prepared
+    std::vector<int> keep, keep_fused;
     std::vector<int> inv;
     // chains of the backward substitution: a chain starts at a root or at a
     // front whose parent has two or more children in the tree part, and
