@@ -54,8 +54,9 @@ __device__ bool bounded_wait(const int* p, int need, int* abort_flag, long long 
 
 // Bounded wait of warp 0 for the children of a unit: lane l polls the
 // completion counters of children l, l + 32, ... (need = their unit count, 1
-// for kWaitOne, their number of units (ti, 0) for kWaitRows), so every child is checked in each round while the other
-// warps of the CTA stay parked at the next barrier. Returns 1 once all are
+// for kWaitOne, their number of units (ti, 0) for kWaitRows), so every child is
+// checked in each round while the other warps of the CTA stay parked at the
+// next barrier. Returns 1 once all are
 // complete, 0 if the wait gave up (the abort flag is then set) or another CTA
 // aborted the kernel. Called by warp 0 only.
 enum { kWaitUnits = 0, kWaitOne = 1, kWaitRows = 2 };
@@ -184,7 +185,7 @@ __device__ __forceinline__ bool panel_f32(const float* M, int Fr, int p0, int pk
 // group): warp 0 factors the panel (pivot columns p0 .. p0 + pk - 1,
 // lane -> row p0 + lane) in registers without a CTA barrier; then every warp
 // applies it to its trailing columns j = p0 + pk + warp + NW c (lane -> row,
-// one shuffle per pivot for the row's U entry, its three columns
+// one shuffle per pivot for the row's U entry, the NC columns of a warp
 // interleaved). Each entry still receives its updates in pivot order with
 // the same roundings as the one-pivot schedule. FULL: pk = 8.
 template <bool FULL, int NW>
@@ -236,7 +237,8 @@ __device__ __forceinline__ void elim_step_f32(float* M, int Fr, int Fc, int p0, 
 // Unit (q, ti, tj) of instance b. Mini front M (Fr x Fc, column-major, ld Fr):
 // rows 0..w-1 / columns 0..w-1 are the pivots, rows w..Fr-1 the contribution
 // rows i0..i0+nr-1, columns w..Fc-1 the contribution columns j0..j0+nc-1.
-// Threads form a 32 x 8 grid (lane -> row, warp -> column).
+// Lane -> row, warp -> column (NW = NT / 32 warps, KC = 32 / NW columns of a
+// thread in the gather).
 //
 // MULTI: the tree parts of several contexts (patterns of different sizes,
 // each possibly batched) in one launch. Tickets 0 .. nu - 1 run through
@@ -425,7 +427,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
             break;
         }
         // ---- children's contributions, in child order for every entry; each
-        // thread holds KC entries of one row and keeps up to 8 loads in
+        // thread holds KC entries of one row and keeps up to 2 KC loads in
         // flight. A warp visits, column by column, only the children that
         // reach the column (a ballot over the children): fronts of the lower
         // tree levels have up to 37 children of a few rows each, and testing
@@ -452,7 +454,7 @@ __device__ __forceinline__ void tree_factor_body(DevSched s_p, TreeSched ts_p, D
                     for (int k = 0; k < KC; ++k) acc[k] = in && jb + NW * k < Fc ? M[i + (jb + NW * k) * Fr] : T(0);
                 }
                 for (int h = 0; h < nk; h += 32) {
-                    if (!ahead)                                    // children h + bit that reach column jb + 8 k
+                    if (!ahead)                                    // children h + bit that reach column jb + NW k
 #pragma unroll
                         for (int k = 0; k < KC; ++k)
                             mk[k] = __ballot_sync(0xffffffffu, jb + NW * k < Fc && h + tx < nk &&
@@ -766,9 +768,6 @@ __device__ __forceinline__ void warp_upper_solve(T* v, const T* U, const T* rcp,
     __syncwarp();
 }
 
-// Front q of instance b (128 threads): gather the pivot entries and the
-// children's contribution vectors, solve with the unit lower pivot block,
-// update the other rows with L21 and leave them as the contribution vector.
 // Forward substitution of front q (already in d, its children in kids) by
 // NT threads: gather the pivot entries and the children's contribution
 // vectors, solve with the unit lower pivot block, update the other rows with
