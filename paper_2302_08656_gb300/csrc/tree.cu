@@ -723,6 +723,16 @@ constexpr auto tree_factor_alone = tree_factor_kernel<T, false, kTreeNtNarrow, s
 // with the 32 unrolled steps of the pivot blocks and fourfold copy loops a
 // separate solve of 25,000 buses took 695 us, rolled 656; refactor_refine
 // 2,003 buses FP32 354 -> 348 us, 70,000 FP64 2784 -> 2737, FP32 1658 -> 1645).
+// STAGED: the panels (forward) or U12 (backward) of the largest front fit the
+// staging buffers (TreeSched::fwd_cstage, bwd_stage). Those kernels are left to
+// the compiler, which holds them to 32 and 40 registers, so that many contexts'
+// CTAs share an SM. The others sum over global memory and need registers for
+// loads in flight: they are bounded to kTreeCtasPerSm CTAs per SM, all that are
+// launched. The two walks of 70,000 buses FP64 with 24 pivots per front took 498
+// + 442 us with the loops unrolled, 831 + 766 rolled, and take 552 + 421 so; the
+// saddle-point solve of 70,000 buses 13.4, 15.0 and 12.3 ms. (All of them
+// bounded: 16 contexts of 2,003 buses FP64, refactorization and solve, 1556 ->
+// 1742 us.)
 //
 // Pivot-block substitutions by one warp (w <= 32), lane i holding entry i in a
 // register and the pivot entry broadcast with a shuffle: the same operations
@@ -951,8 +961,8 @@ __device__ __forceinline__ void bar_sync_staging(int nthr)
 // update sums in pivot order: the results equal a front-by-front substitution
 // bit for bit. Only the chain's top writes its contribution vector and
 // signals completion.
-template <typename T>
-__global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts, DevNum<T> nm0, int B, int* ctr,
+template <typename T, bool STAGED>
+__global__ void __launch_bounds__(128, STAGED ? 0 : kTreeCtasPerSm) tree_fwd_kernel(DevSched s, TreeSched ts, DevNum<T> nm0, int B, int* ctr,
                                                        long long limit)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -964,7 +974,7 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
     const int tid = threadIdx.x, lane = tid & 31;
     const int total = ts.nchains * B;
     int* done = ctr + kCtrHead;
-    const int pw = ts.fwd_cstage ? ts.max_fw : ts.max_w * ts.max_w;    // panel F x w, or pivot block w x w
+    const int pw = STAGED ? ts.max_fw : ts.max_w * ts.max_w;    // panel F x w, or pivot block w x w
     const int ks = ts.fwd_kstage;                               // children's entries staged per front
     const int stage_len = ts.max_w + pw + ks;
     T* vb = reinterpret_cast<T*>(smraw);                        // v of the current and of the previous front
@@ -982,7 +992,7 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
         const T* pan = nm.panel + d.panel_off;
 #pragma unroll 1
         for (int a = me; a < w; a += nthr) cp_word(y + a, nm.vec + d.first + a, (int)sizeof(T));
-        if (ts.fwd_cstage) {
+        if (STAGED) {
 #pragma unroll 1
             for (int c = wi; c < w; c += nw)
 #pragma unroll 1
@@ -1111,7 +1121,7 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
             // warps 1-3 stage the next front while warp 0 solves this one
             if (j + 1 < len && tid >= 32) stage(sb ^ 1, dd[(ds + 1) % 3], nm, 32, 96);
             if (tid < 32) {
-                const int ldp = ts.fwd_cstage ? F : w;
+                const int ldp = STAGED ? F : w;
                 if (w <= 32)
                     warp_lower_solve(v, P, ldp, w);
                 else
@@ -1128,7 +1138,7 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
 #pragma unroll 1
             for (int i = w + tid; i < F; i += 128) {
                 T acc = v[i];
-                if (ts.fwd_cstage)
+                if (STAGED)
 #pragma unroll 4
                     for (int p = 0; p < w; ++p) acc -= P[i + p * F] * v[p];
                 else
@@ -1169,8 +1179,8 @@ __global__ void __launch_bounds__(128) tree_fwd_kernel(DevSched s, TreeSched ts,
 // after it alongside (three descriptor slots). Completion is signalled once,
 // for the last front of the chain: the only front whose children in the tree
 // part are outside it.
-template <typename T>
-__global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts, DevNum<T> nm0, int B, int* ctr,
+template <typename T, bool STAGED>
+__global__ void __launch_bounds__(128, STAGED ? 0 : kTreeCtasPerSm) tree_bwd_kernel(DevSched s, TreeSched ts, DevNum<T> nm0, int B, int* ctr,
                                                        long long limit)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1181,7 +1191,7 @@ __global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts,
     const int tid = threadIdx.x, lane = tid & 31;
     const int total = ts.nchains * B;
     int* done = ctr + kCtrHead + ts.nq * B;                     // after the forward counters
-    const int stage_len = ts.max_w + ts.max_w * ts.max_w + (ts.bwd_stage ? ts.max_wm : 0);
+    const int stage_len = ts.max_w + ts.max_w * ts.max_w + (STAGED ? ts.max_wm : 0);
     T* vb = reinterpret_cast<T*>(smraw);                        // v of the two last fronts: vb, vb + max_F
     T* stg = vb + 2 * ts.max_F;                                 // staging buffers: y, Us, U12s (twice)
     int* rix = reinterpret_cast<int*>(stg + 2 * stage_len);     // index buffers (twice)
@@ -1204,7 +1214,7 @@ __global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts,
         for (int c = wi; c < w; c += nw)
 #pragma unroll 1
             for (int a = lane; a < w; a += 32) cp_word(Us + a + c * w, pan + a + (int64_t)c * F, (int)sizeof(T));
-        if (ts.bwd_stage) {
+        if (STAGED) {
             const T* U12 = pan + (int64_t)F * w;
 #pragma unroll 1
             for (int e = me; e < w * m; e += nthr) cp_word(U12s + e, U12 + e, (int)sizeof(T));
@@ -1271,7 +1281,7 @@ __global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts,
 #pragma unroll 1
                 for (int a = tid; a < w; a += 128) {
                     T acc = y[a];
-                    if (ts.bwd_stage)
+                    if (STAGED)
 #pragma unroll 4
                         for (int tt = 0; tt < m; ++tt) acc -= U12s[a + tt * w] * v[w + tt];
                     else
@@ -1285,7 +1295,7 @@ __global__ void __launch_bounds__(128) tree_bwd_kernel(DevSched s, TreeSched ts,
                 if (tid < G * w) {
                     // in sequence, four terms' loads issued ahead of their FMAs
                     const int a = tid % w, g = tid / w;
-                    const T* Ua = ts.bwd_stage ? U12s + a : U12 + a;
+                    const T* Ua = STAGED ? U12s + a : U12 + a;
                     int tt = g;
                     for (; tt + 3 * G < m; tt += 4 * G) {
                         T u[4], x[4];
@@ -1346,8 +1356,8 @@ cudaError_t tree_grid(int kind, size_t smem, int* grid)
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
     if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_wide<T>, kTreeNt, smem);
     else if (kind == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_factor_multi<T>, kTreeNt, smem);
-    else if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_fwd_kernel<T>, 128, smem);
-    else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_bwd_kernel<T>, 128, smem);
+    else if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_fwd_kernel<T, false>, 128, smem);
+    else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tree_bwd_kernel<T, false>, 128, smem);   // more registers
     if (e != cudaSuccess) return e;
     // at most kTreeCtasPerSm resident CTAs per SM by default (measured: more
     // share an SM's FP64 pipe without hiding more of the dependency waits);
@@ -1399,7 +1409,8 @@ cudaError_t launch_tree_fwd(const DevSched& s, const TreeSched& t, const DevNum<
     const int g = std::min<long long>(grid, (long long)t.nq * batch);
     if (g <= 0) return cudaSuccess;
     if (t.fr == nullptr || t.kid == nullptr) return cudaErrorInvalidValue;
-    tree_fwd_kernel<T><<<g, 128, smem, st>>>(s, t, nm, batch, ctr, spin_limit);
+    const auto kernel = t.fwd_cstage ? tree_fwd_kernel<T, true> : tree_fwd_kernel<T, false>;
+    kernel<<<g, 128, smem, st>>>(s, t, nm, batch, ctr, spin_limit);
     return cudaGetLastError();
 }
 
@@ -1410,7 +1421,8 @@ cudaError_t launch_tree_bwd(const DevSched& s, const TreeSched& t, const DevNum<
     const int g = std::min<long long>(grid, (long long)t.nchains * batch);
     if (g <= 0) return cudaSuccess;
     if (t.fr == nullptr || t.bwd_chain == nullptr || t.bwd_chain_ptr == nullptr) return cudaErrorInvalidValue;
-    tree_bwd_kernel<T><<<g, 128, smem, st>>>(s, t, nm, batch, ctr, spin_limit);
+    const auto kernel = t.bwd_stage ? tree_bwd_kernel<T, true> : tree_bwd_kernel<T, false>;
+    kernel<<<g, 128, smem, st>>>(s, t, nm, batch, ctr, spin_limit);
     return cudaGetLastError();
 }
 
@@ -1447,10 +1459,14 @@ cudaError_t configure_tree_kernels(int optin)
     if ((e = allow_smem_tree(tree_factor_narrow<float>, optin))) return e;
     if ((e = allow_smem_tree(tree_factor_multi<double>, optin))) return e;
     if ((e = allow_smem_tree(tree_factor_multi<float>, optin))) return e;
-    if ((e = allow_smem_tree(tree_fwd_kernel<double>, optin))) return e;
-    if ((e = allow_smem_tree(tree_fwd_kernel<float>, optin))) return e;
-    if ((e = allow_smem_tree(tree_bwd_kernel<double>, optin))) return e;
-    if ((e = allow_smem_tree(tree_bwd_kernel<float>, optin))) return e;
+    if ((e = allow_smem_tree(tree_fwd_kernel<double, false>, optin))) return e;
+    if ((e = allow_smem_tree(tree_fwd_kernel<double, true>, optin))) return e;
+    if ((e = allow_smem_tree(tree_fwd_kernel<float, false>, optin))) return e;
+    if ((e = allow_smem_tree(tree_fwd_kernel<float, true>, optin))) return e;
+    if ((e = allow_smem_tree(tree_bwd_kernel<double, false>, optin))) return e;
+    if ((e = allow_smem_tree(tree_bwd_kernel<double, true>, optin))) return e;
+    if ((e = allow_smem_tree(tree_bwd_kernel<float, false>, optin))) return e;
+    if ((e = allow_smem_tree(tree_bwd_kernel<float, true>, optin))) return e;
     return cudaSuccess;
 }
 
