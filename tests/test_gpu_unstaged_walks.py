@@ -19,16 +19,16 @@ def test_unstaged_panels_keep_their_loads_in_flight():
     pat = KKTPattern(make_grid(1, 70_000))
     vals = torch.from_numpy(pat.values(pat.point(1, 0, 1e-3))).to("cuda:0")
     rhs = torch.from_numpy(pat.rhs(1, 0)).to("cuda:0")
-    us = {}
-    for precision in ("fp32", "fp64"):
-        s = K.KKTSolver(pat.rowptr, pat.colidx, pat.n_primal, precision=precision, max_pivots=24)
+    solvers = {p: K.KKTSolver(pat.rowptr, pat.colidx, pat.n_primal, precision=p, max_pivots=24) for p in ("fp32", "fp64")}
+    for s in solvers.values():
         s.refactor(vals)
         s.set_profiling(True)
-        times = []
-        for _ in range(30):
+    us = dict.fromkeys(solvers, np.inf)
+    for _ in range(30):                                        # in turn, the least of each
+        for p, s in solvers.items():
             s.solve(rhs)
             stats = s.kernel_stats()
-            times.append(stats["tree_fwd_kernel"][1] + stats["tree_bwd_kernel"][1])
-        us[precision] = 1000.0 * float(np.median(times))
+            us[p] = min(us[p], 1000.0 * (stats["tree_fwd_kernel"][1] + stats["tree_bwd_kernel"][1]))
+    for s in solvers.values():
         s.close()
     assert us["fp64"] <= 2.5 * us["fp32"], us
